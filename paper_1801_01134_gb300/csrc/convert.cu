@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(256) k_validate_cols(int64_t n, int64_t m, int
     const int64_t j = base + k * 32 + lane;
     const int32_t col = j < end ? colidx[j] : 0;
     int32_t prev = __shfl_up_sync(0xffffffffu, col, 1);
-    if (lane == 0) prev = j > 0 ? colidx[j - 1] : 0;
+    if (lane == 0) prev = j > 0 && j < end ? colidx[j - 1] : 0;  // nothing past the array is read
     if (j < end) {
       const int o = (int)(j - base);
       const bool row_start = (st[o >> 5] >> (o & 31)) & 1u;
