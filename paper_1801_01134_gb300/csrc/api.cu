@@ -571,20 +571,7 @@ spc5_status spc5_select(int64_t n, int64_t m, int64_t nnz, const int64_t* rowptr
       for (int q = 0; q < 16; ++q)
         xin[q] = (float)((std::log1p(f[q]) - (double)model->feat_mean[q]) /
                          (double)(model->feat_scale[q] != 0.f ? model->feat_scale[q] : 1.f));
-      void* buf = nullptr;
-      cudaError_t e = cudaMalloc(&buf, sizeof(float) * 28);
-      if (e == cudaSuccess) e = cudaMemcpyAsync(buf, xin, sizeof(xin), cudaMemcpyHostToDevice, s);
-      if (e != cudaSuccess) {
-        cudaFree(buf);
-        return cuda_fail(e, "select: MLP input");
-      }
-      st = mlp_infer_impl(model->mlp_params_d, (const float*)buf, 1, (float*)buf + 16, s);
-      if (st == SPC5_OK) {
-        e = cudaMemcpyAsync(score, (float*)buf + 16, sizeof(float) * 12, cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess) st = cuda_fail(e, "select: MLP output");
-      }
-      cudaFree(buf);
+      st = mlp_score_impl(model->mlp_params_d, xin, score, s);
       if (st != SPC5_OK) return st;
       for (int q = 1; q < 12; ++q)
         if (score[q] < score[best]) best = q;

@@ -164,6 +164,7 @@ spc5_status mlp_train_impl(float* P, const float* X, const float* Y, const float
 spc5_status mlp_grad_impl(const float* P, const float* X, const float* Y, const float* M, int B, float* loss,
                           float* grad, cudaStream_t s, int nfeat = 16);
 spc5_status mlp_infer_impl(const float* P, const float* X, int N, float* out, cudaStream_t s, int nfeat = 16);
+spc5_status mlp_score_impl(const float* P, const float* x, float* scores, cudaStream_t s);
 // extended selection features (16 + x-access locality, short rows, SM fraction)
 spc5_status features_ext_impl(int64_t n, int64_t nnz, const int64_t* rowptr, const int32_t* colidx,
                               double sm_frac, double* f, cudaStream_t s);

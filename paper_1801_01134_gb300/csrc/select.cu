@@ -158,38 +158,70 @@ __global__ void __launch_bounds__(kStepThreads) k_mlp_step(float* __restrict__ P
   }
 }
 
-// scores of N samples: one thread per (sample, output); hidden layers of a
-// sample recomputed per output is wasteful but N is small; instead one thread
-// per sample with the activations in local arrays
+// Scores of N samples, a thread block per sample: 64 threads, one per hidden
+// unit, the activations in shared memory; every sum runs over its inputs in
+// order. One sample (spc5_select) is bound by the latency of its three layers:
+// one thread working through all of them alone took 161 us, the block 5.
 template <int NF>
-__global__ void __launch_bounds__(128) k_mlp_infer(const float* __restrict__ P, const float* __restrict__ X, int N,
-                                                   float* __restrict__ out) {
+struct MlpInput {
+  float v[NF];
+};
+
+template <int NF>
+__device__ __forceinline__ void mlp_forward(const float* __restrict__ P, const float* __restrict__ x,
+                                            float* __restrict__ out) {
   constexpr int oW1 = Mlp<NF>::oW1, ob1 = Mlp<NF>::ob1, oW2 = Mlp<NF>::oW2, ob2 = Mlp<NF>::ob2, oW3 = Mlp<NF>::oW3,
-                ob3 = Mlp<NF>::ob3, kNF = NF;
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= N) return;
-  float a1[kH], a2[kH];
-  for (int j = 0; j < kH; ++j) {
-    float a = P[ob1 + j];
-    for (int q = 0; q < kNF; ++q) a = fmaf(P[oW1 + j * kNF + q], X[(int64_t)s * kNF + q], a);
-    a1[j] = a > 0.f ? a : 0.f;
+                ob3 = Mlp<NF>::ob3;
+  __shared__ float a1[kH], a2[kH];
+  const int j = threadIdx.x;
+  float a = P[ob1 + j];
+#pragma unroll
+  for (int q = 0; q < NF; ++q) a = fmaf(P[oW1 + j * NF + q], x[q], a);
+  a1[j] = a > 0.f ? a : 0.f;
+  __syncthreads();
+  a = P[ob2 + j];
+#pragma unroll
+  for (int q = 0; q < kH; ++q) a = fmaf(P[oW2 + j * kH + q], a1[q], a);
+  a2[j] = a > 0.f ? a : 0.f;
+  __syncthreads();
+  if (j < kNO) {
+    a = P[ob3 + j];
+#pragma unroll
+    for (int q = 0; q < kH; ++q) a = fmaf(P[oW3 + j * kH + q], a2[q], a);
+    out[j] = a;
   }
-  for (int j = 0; j < kH; ++j) {
-    float a = P[ob2 + j];
-    for (int q = 0; q < kH; ++q) a = fmaf(P[oW2 + j * kH + q], a1[q], a);
-    a2[j] = a > 0.f ? a : 0.f;
-  }
-  for (int o = 0; o < kNO; ++o) {
-    float a = P[ob3 + o];
-    for (int q = 0; q < kH; ++q) a = fmaf(P[oW3 + o * kH + q], a2[q], a);
-    out[(int64_t)s * kNO + o] = a;
-  }
+}
+
+template <int NF>
+__global__ void __launch_bounds__(kH) k_mlp_infer(const float* __restrict__ P, const float* __restrict__ X,
+                                                  float* __restrict__ out) {
+  mlp_forward<NF>(P, X + (int64_t)blockIdx.x * NF, out + (int64_t)blockIdx.x * kNO);
+}
+
+// one sample, its inputs passed with the launch
+template <int NF>
+__global__ void __launch_bounds__(kH) k_mlp_infer_one(const float* __restrict__ P, const MlpInput<NF> x,
+                                                      float* __restrict__ out) {
+  mlp_forward<NF>(P, x.v, out);
 }
 
 struct DBuf {
   void* p = nullptr;
   ~DBuf() {
     if (p) cudaFree(p);
+  }
+};
+
+// scratch from the library's pool, given back in the order of its stream
+struct PoolBuf {
+  void* p = nullptr;
+  cudaStream_t s = nullptr;
+  cudaError_t alloc(size_t bytes, cudaStream_t st) {
+    s = st;
+    return pool_alloc(&p, bytes, st);
+  }
+  ~PoolBuf() {
+    if (p) cudaFreeAsync(p, s);
   }
 };
 
@@ -231,8 +263,8 @@ bool lstsq(std::vector<double> V, std::vector<double> y, int N, int k, double* c
 
 spc5_status features_impl(int64_t n, int64_t nnz, const int64_t* rowptr, const int32_t* colidx, double* f,
                           cudaStream_t s) {
-  DBuf acc;
-  cudaError_t e = cudaMalloc(&acc.p, sizeof(unsigned long long) * 16);
+  PoolBuf acc;
+  cudaError_t e = acc.alloc(sizeof(unsigned long long) * 16, s);
   if (e == cudaSuccess) e = launch_block_counts(n, nnz, rowptr, colidx, (unsigned long long*)acc.p, s);
   unsigned long long h[15];
   if (e == cudaSuccess) e = cudaMemcpyAsync(h, acc.p, sizeof(h), cudaMemcpyDeviceToHost, s);
@@ -281,8 +313,8 @@ spc5_status features_ext_impl(int64_t n, int64_t nnz, const int64_t* rowptr, con
                               double sm_frac, double* f, cudaStream_t s) {
   spc5_status st = features_impl(n, nnz, rowptr, colidx, f, s);
   if (st != SPC5_OK) return st;
-  DBuf acc;
-  cudaError_t e = cudaMalloc(&acc.p, sizeof(unsigned long long) * 2);
+  PoolBuf acc;
+  cudaError_t e = acc.alloc(sizeof(unsigned long long) * 2, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(acc.p, 0, sizeof(unsigned long long) * 2, s);
   if (e == cudaSuccess && n > 0) {
     const int64_t warps = (n + 31) / 32;
@@ -379,10 +411,26 @@ spc5_status mlp_grad_impl(const float* P, const float* X, const float* Y, const 
 
 spc5_status mlp_infer_impl(const float* P, const float* X, int N, float* out, cudaStream_t s, int nfeat) {
   if (nfeat != 16 && nfeat != 20) return fail(SPC5_EINVAL, "mlp_infer: nfeat must be 16 or 20");
-  if (N > 0 && nfeat == 16) k_mlp_infer<16><<<(unsigned)((N + 127) / 128), 128, 0, s>>>(P, X, N, out);
-  if (N > 0 && nfeat == 20) k_mlp_infer<20><<<(unsigned)((N + 127) / 128), 128, 0, s>>>(P, X, N, out);
+  if (N > 0 && nfeat == 16) k_mlp_infer<16><<<(unsigned)N, kH, 0, s>>>(P, X, out);
+  if (N > 0 && nfeat == 20) k_mlp_infer<20><<<(unsigned)N, kH, 0, s>>>(P, X, out);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "mlp_infer");
+  return SPC5_OK;
+}
+
+// scores (host) of one sample with 16 inputs (host); synchronises s
+spc5_status mlp_score_impl(const float* P, const float* x, float* scores, cudaStream_t s) {
+  MlpInput<kNF> in;
+  for (int q = 0; q < kNF; ++q) in.v[q] = x[q];
+  PoolBuf out;
+  cudaError_t e = out.alloc(sizeof(float) * kNO, s);
+  if (e == cudaSuccess) {
+    k_mlp_infer_one<kNF><<<1, kH, 0, s>>>(P, in, (float*)out.p);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaMemcpyAsync(scores, out.p, sizeof(float) * kNO, cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) return cuda_fail(e, "select: MLP scores");
   return SPC5_OK;
 }
 
