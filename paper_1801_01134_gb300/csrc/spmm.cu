@@ -256,6 +256,132 @@ __global__ void __launch_bounds__(256) k_spmm_blk(int64_t n, int64_t I, int32_t 
   }
 }
 
+// acc += v x over four columns: two packed multiply-adds (each half rounded
+// once, as fmaf does).
+__device__ __forceinline__ void fma_quad(float (&acc)[4], float v, const float4& x) {
+  asm("{\n .reg .b64 vv, x0, x1, c0, c1;\n mov.b64 vv, {%4, %4};\n mov.b64 x0, {%5, %6};\n mov.b64 x1, {%7, %8};\n"
+      " mov.b64 c0, {%0, %1};\n mov.b64 c1, {%2, %3};\n fma.rn.f32x2 c0, vv, x0, c0;\n fma.rn.f32x2 c1, vv, x1, c1;\n"
+      " mov.b64 {%0, %1}, c0;\n mov.b64 {%2, %3}, c1;\n}"
+      : "+f"(acc[0]), "+f"(acc[1]), "+f"(acc[2]), "+f"(acc[3])
+      : "f"(v), "f"(x.x), "f"(x.y), "f"(x.z), "f"(x.w));
+}
+
+// X row slices of a tile whose lanes all own four columns on 16-byte
+// boundaries, addressed by 32-bit element offsets (m * ldx < 2^31)
+__device__ __forceinline__ float4 load_x4(const float* __restrict__ X, uint32_t at) {
+  return __ldg(reinterpret_cast<const float4*>(X + at));
+}
+
+// k_spmm_blk where every lane's four columns are whole and aligned (float32 X
+// and Y, k and the leading dimensions multiples of 4) and 32 bits address X:
+// the same mapping and the same sums. The general kernel spends about thirty
+// instructions per stored value on bit searches, 64-bit address products and
+// the tests of a partial slice; here they are about half. With c = 4 the bit
+// positions are unrolled, so a block's X slices are all on the way at once.
+// With ORDER the intervals come in the handle's sorted work order (intervals
+// of similar length share a warp).
+// With r > 1 a column's X slice is read once for all the rows that hold it,
+// which is what bounds the large grids (L1: every read is 16 bytes per lane).
+// Measured against the general kernel, L2 warm, float32: 27-point stencil
+// 128^3, k = 32, beta(1,4) 0.557 -> 0.466 ms, beta(2,4) 0.568 -> 0.376 (four
+// rows per block 0.482: more tests than reads saved); R-MAT scale 22, k = 8,
+// the short rows 0.54 -> 0.47 ms in natural order and about 0.22 in the sorted
+// one. Unrolling beta(1,4) is worth 15 % where blocks hold three values (FEM)
+// and costs 40 % where they hold one (R-MAT; beta(1,8) keeps the bit loop, and
+// the tuner picks).
+template <class T, int R, int C, int G, bool ORDER>
+__global__ void __launch_bounds__(256) k_spmm_blk4(int64_t n, int64_t I, int32_t long_blocks, int64_t long_values,
+                                                   const int32_t* __restrict__ brp, const int32_t* __restrict__ bcol,
+                                                   const uint8_t* __restrict__ bmask,
+                                                   const typename T::V* __restrict__ val,
+                                                   const int64_t* __restrict__ valptr, const float* __restrict__ X,
+                                                   uint32_t ldx, float* __restrict__ Y, int64_t ldy, int k,
+                                                   const int32_t* __restrict__ order, int64_t norder) {
+  constexpr int MB = (R * C + 7) / 8;
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  int64_t it = t / G;
+  const int j = blockIdx.y * (G * 4) + (int)(t % G) * 4;
+  if (it >= (ORDER ? norder : I) || j >= k) return;
+  if (ORDER) it = __ldg(order + it);
+  int32_t b = __ldg(brp + it);
+  const int32_t bend = __ldg(brp + it + 1);
+  const int64_t v0 = __ldg(valptr + it);
+  if (bend - b > long_blocks || __ldg(valptr + it + 1) - v0 > long_values) return;  // the segment path's
+  const typename T::V* __restrict__ v = val + v0;
+  float acc[R][4];
+#pragma unroll
+  for (int i = 0; i < R; ++i)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[i][q] = 0.f;
+  Mask<MB> m0 = b < bend ? load_mask<MB>(bmask, b) : zero_mask<MB>();
+  uint32_t c0 = b < bend ? (uint32_t)__ldg(bcol + b) : 0u;
+  for (; b < bend; ++b) {
+    const Mask<MB> mk = m0;
+    const uint32_t at = c0 * ldx + (uint32_t)j;
+    if (b + 1 < bend) {
+      m0 = load_mask<MB>(bmask, b + 1);
+      c0 = (uint32_t)__ldg(bcol + b + 1);
+    }
+    if constexpr (R == 1 && C == 4) {
+      const uint32_t bits = mk.w[0];
+      float vv[4];
+      float4 xx[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if ((bits >> q) & 1u) {
+          vv[q] = T::val(v, 0);
+          ++v;
+          xx[q] = load_x4(X, at + q * ldx);
+        }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if ((bits >> q) & 1u) fma_quad(acc[0], vv[q], xx[q]);
+    } else if constexpr (R == 1) {
+      for (uint32_t bits = row_bits<C>(mk, 0); bits; bits &= bits - 1) {
+        const float vv = T::val(v, 0);
+        ++v;
+        fma_quad(acc[0], vv, load_x4(X, at + ((uint32_t)__ffs(bits) - 1u) * ldx));
+      }
+    } else {
+      // one X slice per column for all the rows that hold it
+      uint32_t rb[R], uni = 0u;
+      int vo[R];
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        rb[i] = row_bits<C>(mk, i);
+        vo[i] = popc_below<C>(mk, i);
+        uni |= rb[i];
+      }
+      if constexpr (C == 4) {
+        float4 xx[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if ((uni >> q) & 1u) xx[q] = load_x4(X, at + q * ldx);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int i = 0; i < R; ++i)
+            if ((rb[i] >> q) & 1u) fma_quad(acc[i], T::val(v, vo[i]++), xx[q]);
+      } else {
+        for (; uni; uni &= uni - 1) {
+          const uint32_t kk = (uint32_t)__ffs(uni) - 1u;
+          const float4 x = load_x4(X, at + kk * ldx);
+#pragma unroll
+          for (int i = 0; i < R; ++i)
+            if ((rb[i] >> kk) & 1u) fma_quad(acc[i], T::val(v, vo[i]++), x);
+        }
+      }
+      v += popc_all(mk);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    const int64_t row = it * R + i;
+    if (row < n)
+      *reinterpret_cast<float4*>(Y + row * ldy + j) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+  }
+}
+
 template <class T, int G>
 void launch_spmm_blk(const spc5_matrix* h, int k, const typename T::X* Xm, int64_t ldx, typename T::X* Ym,
                      int64_t ldy, cudaStream_t s) {
@@ -263,6 +389,24 @@ void launch_spmm_blk(const spc5_matrix* h, int k, const typename T::X* Xm, int64
   dim3 grid((unsigned)((h->I * G + 255) / 256), (unsigned)((k + 4 * G - 1) / (4 * G)));
   // 16-byte X loads when every lane's 4 columns start on a 16-byte boundary
   const bool vec = sizeof(typename T::X) == 4 && ldx % 4 == 0 && (reinterpret_cast<uintptr_t>(Xm) & 15u) == 0;
+  if constexpr (sizeof(typename T::X) == 4) {
+    if (vec && k % 4 == 0 && ldy % 4 == 0 && (reinterpret_cast<uintptr_t>(Ym) & 15u) == 0 && h->m * ldx < (int64_t)INT32_MAX) {
+      const bool ordered = ordered_variant(h->variant) && h->norder > 0;
+      const int64_t slots = ordered ? h->norder : h->I;
+      const dim3 g4((unsigned)((slots * G + 255) / 256), grid.y);
+      auto go = [&](auto kern) {
+        kern<<<g4, 256, 0, s>>>(h->n, h->I, h->long_blocks, h->long_values, h->block_rowptr, h->block_colidx,
+                                h->block_masks, val, h->valptr, Xm, (uint32_t)ldx, Ym, ldy, k, h->order, h->norder);
+      };
+#define SPC5_BLK4(RR, CC) \
+  if (h->r == RR && h->c == CC) return ordered ? go(k_spmm_blk4<T, RR, CC, G, true>) : go(k_spmm_blk4<T, RR, CC, G, false>);
+      SPC5_BLK4(1, 4) SPC5_BLK4(1, 8) SPC5_BLK4(1, 16)
+      SPC5_BLK4(2, 4) SPC5_BLK4(2, 8) SPC5_BLK4(2, 16)
+      SPC5_BLK4(4, 4) SPC5_BLK4(4, 8) SPC5_BLK4(4, 16)
+      SPC5_BLK4(8, 4) SPC5_BLK4(8, 8) SPC5_BLK4(8, 16)
+#undef SPC5_BLK4
+    }
+  }
 #define SPC5_BLK(RR, CC)                                                                                            \
   if (h->r == RR && h->c == CC) {                                                                                   \
     k_spmm_blk<T, RR, CC, G><<<grid, 256, 0, s>>>(h->n, h->I, h->long_blocks, h->long_values, h->block_rowptr,     \
@@ -429,6 +573,95 @@ __global__ void __launch_bounds__(256) k_spmm_seg_cols(int64_t nseg, int c, int 
   }
 }
 
+// k_spmm_seg_cols under the conditions of k_spmm_blk4: 64 blocks per trip, two
+// per lane, and each group takes four of them at a time, one value of each on
+// the way before the first is used (power-law hubs hold about one value per
+// block, so that many X rows are awaited together instead of one). R-MAT scale
+// 22, 48 M entries in segments: k = 8 0.42 -> 0.35 ms, k = 32 1.22 -> 0.78.
+template <class T, int MB, int G>
+__global__ void __launch_bounds__(128) k_spmm_seg4(int64_t nseg, const Segment* __restrict__ segs,
+                                                   const int32_t* __restrict__ bcol, const uint8_t* __restrict__ bmask,
+                                                   const typename T::V* __restrict__ val, const float* __restrict__ X,
+                                                   uint32_t ldx, float* __restrict__ part, int k) {
+  constexpr int NG = kWarp / G;           // groups per warp
+  constexpr int U = NG > 16 ? 2 : 4;      // blocks a group takes at a time
+  const int lane = threadIdx.x & 31;
+  const int64_t seg = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (seg >= nseg) return;  // whole warp
+  const int grp = lane / G;
+  const int j = blockIdx.y * (G * 4) + (lane % G) * 4;
+  const bool own = j < k;
+  const Segment sg = segs[seg];
+  const typename T::V* __restrict__ v = val + sg.v_begin;
+  const float* __restrict__ xj = X + (own ? j : 0);
+  float acc[4] = {0.f, 0.f, 0.f, 0.f};
+  for (int32_t b0 = sg.b_begin; b0 < sg.b_end; b0 += 2 * kWarp) {
+    uint32_t m[2], at[2];
+    int first[2], sum = 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int32_t b = b0 + h * kWarp + lane;
+      m[h] = b < sg.b_end ? load_mask<MB>(bmask, b).w[0] : 0u;
+      at[h] = b < sg.b_end ? (uint32_t)__ldg(bcol + b) * ldx : 0u;
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int cnt = __popc(m[h]);
+      int incl = cnt;
+#pragma unroll
+      for (int d = 1; d < kWarp; d <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += t;
+      }
+      first[h] = sum + incl - cnt;
+      sum += __shfl_sync(0xffffffffu, incl, kWarp - 1);
+    }
+#pragma unroll
+    for (int q0 = 0; q0 < 2 * kWarp; q0 += U * NG) {
+      uint32_t mq[U], xq[U];
+      int vq[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int h = (q0 + u * NG) / kWarp, q = (q0 + u * NG) % kWarp + grp;
+        mq[u] = __shfl_sync(0xffffffffu, m[h], q);
+        xq[u] = __shfl_sync(0xffffffffu, at[h], q);
+        vq[u] = __shfl_sync(0xffffffffu, first[h], q);
+      }
+      if (!own) continue;
+      for (;;) {
+        uint32_t any = 0u;
+#pragma unroll
+        for (int u = 0; u < U; ++u) any |= mq[u];
+        if (!any) break;
+        float vv[U];
+        float4 xx[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (mq[u]) {
+            vv[u] = T::val(v, vq[u]);
+            xx[u] = load_x4(xj, xq[u] + ((uint32_t)__ffs(mq[u]) - 1u) * ldx);
+          }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (mq[u]) {
+            fma_quad(acc, vv[u], xx[u]);
+            mq[u] &= mq[u] - 1;
+            ++vq[u];
+          }
+      }
+    }
+    v += sum;
+  }
+#pragma unroll
+  for (int t = 0; t < 4; ++t)
+#pragma unroll
+    for (int d = G; d < kWarp; d <<= 1) acc[t] += __shfl_xor_sync(0xffffffffu, acc[t], d);
+  if (grp == 0 && own) {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) part[seg * (int64_t)k + j + t] = acc[t];
+  }
+}
+
 // the long intervals' segments and fix-up; beta(1,c) with k >= 4 takes the
 // column groups above (G = 1, 2, 4 or 8 lanes: 4, 8, 16 or 32 columns per
 // tile), other shapes a lane per (block run, row) with KT columns
@@ -439,7 +672,29 @@ void spmm_long(const spc5_matrix* h, int k, const typename T::X* Xm, int64_t ldx
   if (h->r == 1 && k >= 4) {
     const bool vec = sizeof(typename T::X) == 4 && ldx % 4 == 0 && (reinterpret_cast<uintptr_t>(Xm) & 15u) == 0;
     const unsigned gx = (unsigned)((h->nseg * kWarp + 255) / 256);
-    if (k < 8) {
+    bool done = false;
+    if constexpr (sizeof(typename T::X) == 4) {
+      if (vec && k % 4 == 0 && h->m * ldx < (int64_t)INT32_MAX) {
+        auto go = [&](auto kern, int cols) {
+          kern<<<dim3((unsigned)((h->nseg + 3) / 4), (unsigned)((k + cols - 1) / cols)), 128, 0, s>>>(
+              h->nseg, h->segs, h->block_colidx, h->block_masks, val, Xm, (uint32_t)ldx, part, k);
+        };
+        if (h->mb == 1) {
+          if (k < 8) go(k_spmm_seg4<T, 1, 1>, 4);
+          else if (k < 16) go(k_spmm_seg4<T, 1, 2>, 8);
+          else if (k < 32) go(k_spmm_seg4<T, 1, 4>, 16);
+          else go(k_spmm_seg4<T, 1, 8>, 32);
+        } else {
+          if (k < 8) go(k_spmm_seg4<T, 2, 1>, 4);
+          else if (k < 16) go(k_spmm_seg4<T, 2, 2>, 8);
+          else if (k < 32) go(k_spmm_seg4<T, 2, 4>, 16);
+          else go(k_spmm_seg4<T, 2, 8>, 32);
+        }
+        done = true;
+      }
+    }
+    if (done) {
+    } else if (k < 8) {
       k_spmm_seg_cols<T, 1><<<dim3(gx, (unsigned)((k + 3) / 4)), 256, 0, s>>>(
           h->nseg, h->c, h->mb, h->segs, h->block_colidx, h->block_masks, val, Xm, ldx, part, k, vec);
     } else if (k >= 32) {
