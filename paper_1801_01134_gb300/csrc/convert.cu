@@ -788,15 +788,20 @@ __global__ void k_scan_apply(const int32_t* __restrict__ in, int64_t L, const in
 // hands the kept memory back.
 constexpr int kMaxPoolDevices = 64;
 std::mutex g_pool_mu;
-cudaMemPool_t g_pools[kMaxPoolDevices] = {};
+// Two pools per device: the arenas have one of their own. Scratch carved out
+// of an arena's freed place leaves it too small for the next arena, and the
+// pool then maps new memory (about a tenth of the conversions of a series
+// paid 5 ms).
+enum PoolKind { kScratchPool = 0, kArenaPool = 1, kPoolKinds = 2 };
+cudaMemPool_t g_pools[kMaxPoolDevices][kPoolKinds] = {};
 
-cudaError_t handle_pool(cudaMemPool_t* out) {
+cudaError_t handle_pool(cudaMemPool_t* out, PoolKind kind = kScratchPool) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= kMaxPoolDevices) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lock(g_pool_mu);
-  if (!g_pools[dev]) {
+  if (!g_pools[dev][kind]) {
     cudaMemPoolProps props = {};
     props.allocType = cudaMemAllocationTypePinned;
     props.location.type = cudaMemLocationTypeDevice;
@@ -810,9 +815,9 @@ cudaError_t handle_pool(cudaMemPool_t* out) {
       cudaMemPoolDestroy(p);
       return e;
     }
-    g_pools[dev] = p;
+    g_pools[dev][kind] = p;
   }
-  *out = g_pools[dev];
+  *out = g_pools[dev][kind];
   return cudaSuccess;
 }
 
@@ -939,7 +944,7 @@ cudaError_t alloc_arena(spc5_matrix* h, int64_t nb, int64_t nnz, int64_t ns, cud
   }
   uint8_t* base = nullptr;
   cudaMemPool_t pool = nullptr;
-  cudaError_t e = handle_pool(&pool);
+  cudaError_t e = handle_pool(&pool, kArenaPool);
   if (e == cudaSuccess) e = cudaMallocFromPoolAsync((void**)&base, total, pool, s);
   if (e != cudaSuccess) return e;
   h->arena = base;
@@ -1327,10 +1332,11 @@ cudaError_t trim_pools() {
   std::lock_guard<std::mutex> lock(g_pool_mu);
   cudaError_t e = cudaSuccess;
   for (int d = 0; d < kMaxPoolDevices; ++d)
-    if (g_pools[d]) {
-      const cudaError_t e2 = cudaMemPoolTrimTo(g_pools[d], 0);
-      if (e == cudaSuccess) e = e2;
-    }
+    for (cudaMemPool_t p : g_pools[d])
+      if (p) {
+        const cudaError_t e2 = cudaMemPoolTrimTo(p, 0);
+        if (e == cudaSuccess) e = e2;
+      }
   return e;
 }
 
