@@ -237,9 +237,16 @@ __global__ void __launch_bounds__(256) k_batch(const MatDesc* __restrict__ mats,
       const int64_t row = it * r + i;
       if (row < d.n) static_cast<X*>(d.y)[row] = acc;
     } else {
-      // one warp per segment, cut into 32/r contiguous runs, lane = (run,
-      // row), the same sums in the same order as k_spmv_segments
+      // one warp per segment, the same sums in the same order as
+      // k_spmv_segments: r = 1 streamed, else cut into 32/r contiguous runs,
+      // lane = (run, row)
       const Segment sg = d.segs[itm.i0];
+      if (r == 1) {
+        const A sum = mb == 1 ? segment_sum_r1<1, T>(sg, d.bcol, d.bmask, val, x)
+                              : segment_sum_r1<2, T>(sg, d.bcol, d.bmask, val, x);
+        if (lane == 0) static_cast<A*>(d.partials)[itm.i0] = sum;
+        continue;
+      }
       const int S = kWarp >> d.log2r;
       const int slot = lane >> d.log2r, i = lane & (r - 1);
       const int32_t per = (sg.b_end - sg.b_begin + S - 1) / S;

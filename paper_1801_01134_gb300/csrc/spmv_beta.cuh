@@ -743,7 +743,79 @@ __global__ void __launch_bounds__(256) k_spmv_rows_t(int64_t n, int64_t I, int32
 }
 
 // -------------------------------------------------------- long intervals
-// A warp per segment (at most seg_blocks blocks of one long interval). The
+// A segment of a beta(1,c) row: the warp streams its blocks, 64 per trip, two
+// per lane (b and b + 32): mask and column reads are consecutive over the
+// warp, one packed scan of the popcounts places both blocks' values, and every
+// lane adds its blocks' products set bit by set bit (power-law hubs hold about
+// one value per block). All blocks belong to one row, so the lanes' sums meet
+// only at the end, in a fixed tree. The sum (in every lane) depends only on the
+// segment. Lanes walking runs of their own read 32 separate places per
+// instruction, three times per value (mask windows aside), where this reads
+// scattered x entries only: R-MAT scale 22, 48 of 65 M entries in segments,
+// whole product (float64, beta(1,4), variant 30) 0.425 -> 0.382 ms.
+template <int MB, class T>
+__device__ __forceinline__ typename T::A segment_sum_r1(const Segment& sg, const int32_t* __restrict__ bcol,
+                                                        const uint8_t* __restrict__ bmask,
+                                                        const typename T::V* __restrict__ val,
+                                                        const typename T::X* __restrict__ x) {
+  using A = typename T::A;
+  constexpr unsigned kAll = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const typename T::V* __restrict__ v = val + sg.v_begin;
+  A acc0 = 0, acc1 = 0;
+  int32_t b = sg.b_begin + lane;
+  uint32_t n0 = b < sg.b_end ? load_mask<MB>(bmask, b).w[0] : 0u;
+  uint32_t n1 = b + 32 < sg.b_end ? load_mask<MB>(bmask, b + 32).w[0] : 0u;
+  int32_t d0 = b < sg.b_end ? __ldg(bcol + b) : 0, d1 = b + 32 < sg.b_end ? __ldg(bcol + b + 32) : 0;
+  for (int32_t t = sg.b_begin; t < sg.b_end; t += 64) {
+    uint32_t m0 = n0, m1 = n1;
+    const int32_t c0 = d0, c1 = d1;
+    b += 64;  // the next trip's blocks
+    n0 = b < sg.b_end ? load_mask<MB>(bmask, b).w[0] : 0u;
+    n1 = b + 32 < sg.b_end ? load_mask<MB>(bmask, b + 32).w[0] : 0u;
+    d0 = b < sg.b_end ? __ldg(bcol + b) : 0;
+    d1 = b + 32 < sg.b_end ? __ldg(bcol + b + 32) : 0;
+    const int own = __popc(m0) | (__popc(m1) << 16);
+    int incl = own;
+#pragma unroll
+    for (int d = 1; d < kWarp; d <<= 1) {
+      const int u = __shfl_up_sync(kAll, incl, d);
+      if (lane >= d) incl += u;
+    }
+    const int all = __shfl_sync(kAll, incl, kWarp - 1);
+    const int before = incl - own;
+    int v0 = before & 0xffff, v1 = (all & 0xffff) + (before >> 16);
+    while (m0 | m1) {
+      A a0 = 0, x0 = 0, a1 = 0, x1 = 0;
+      if (m0) {
+        a0 = T::val(v, v0);
+        x0 = T::xv(x, (int64_t)c0 + __ffs(m0) - 1);
+      }
+      if (m1) {
+        a1 = T::val(v, v1);
+        x1 = T::xv(x, (int64_t)c1 + __ffs(m1) - 1);
+      }
+      if (m0) {
+        acc0 = fmadd<T>(a0, x0, acc0);
+        m0 &= m0 - 1;
+        ++v0;
+      }
+      if (m1) {
+        acc1 = fmadd<T>(a1, x1, acc1);
+        m1 &= m1 - 1;
+        ++v1;
+      }
+    }
+    v += (all & 0xffff) + (all >> 16);
+  }
+  A acc = acc0 + acc1;
+#pragma unroll
+  for (int d = kWarp / 2; d >= 1; d >>= 1) acc += __shfl_xor_sync(kAll, acc, d);
+  return acc;
+}
+
+// A warp per segment (at most seg_blocks blocks of one long interval; r = 1 is
+// streamed, see segment_sum_r1). The
 // segment's blocks are cut into S = 32/r contiguous runs, one per group of r
 // lanes (lane = run slot, row i). A first pass counts the stored values of
 // each run from its masks and a shuffle scan over the slots gives every run
@@ -764,8 +836,13 @@ __device__ __forceinline__ void segments_body(int64_t bid, int64_t nseg, const S
   const int lane = threadIdx.x & 31;
   const int64_t seg = (bid * blockDim.x + threadIdx.x) >> 5;
   if (seg >= nseg) return;  // whole warp leaves together
-  const int slot = lane / R, i = lane % R;
   const Segment sg = segs[seg];
+  if constexpr (R == 1) {
+    const typename T::A sum = segment_sum_r1<MB, T>(sg, bcol, bmask, val, x);
+    if (lane == 0) partials[seg] = sum;
+    return;
+  }
+  const int slot = lane / R, i = lane % R;
   const int32_t per = (sg.b_end - sg.b_begin + S - 1) / S;
   const int32_t rb = min(sg.b_begin + slot * per, sg.b_end);
   const int32_t re = min(rb + per, sg.b_end);
