@@ -108,8 +108,9 @@ typedef struct {
    *           built when the variant is selected): a row whose blocks all
    *           hold one value is read like a two-lane CSR row (no mask read);
    *           the same sums as 22, bit for bit.
-   * spc5_cg uses the decode of 16 or 18 when its handle has that variant,
-   * the flattened one otherwise.
+   * spc5_cg unpacks the rows of a matrix without long intervals, whatever
+   * its variant (the products in the order of 0-19); the others' products are
+   * the variant's.
    * Variants 0-19, 30 and 31 compute the same sums in the same order per
    * row, and so do 22 and 33; every variant repeats its own results bit for
    * bit. */
@@ -273,8 +274,8 @@ spc5_status spc5_device_peaks(double* hbm_gbs_out, int* sm_count_out, int* sm_cl
 
 /* spc5_destroy - free the handle and its device arrays (synchronises the
  * device first so that no queued kernel still reads them). NULL is allowed.
- * The arrays of converted handles go back to a memory pool of the library's
- * own (one per device), which keeps them for the next conversion instead of
+ * The arrays of converted handles go back to memory pools of the library's
+ * own (per device), which keep them for the next conversion instead of
  * returning them to the driver; see spc5_pool_trim. */
 spc5_status spc5_destroy(spc5_handle h);
 
