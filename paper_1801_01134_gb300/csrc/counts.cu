@@ -76,6 +76,11 @@ struct CountCut {  // where the range starts: the first column, or INT_MAX, and 
 // ranges of a long group of `total` entries
 __host__ __device__ __forceinline__ int64_t pieces_of(int64_t total) { return (total + kPiece - 1) / kPiece; }
 
+// Column b starts a new run after a: they lie at least 16 apart. Unsigned, so
+// that the whole range [-16, 2^31) works (-16 stands before a list's first
+// column).
+__device__ __forceinline__ bool apart(int32_t a, int32_t b) { return (uint32_t)b - (uint32_t)a >= 16u; }
+
 // lists before level k's in CountShared::open
 __device__ __forceinline__ int open_base(int k) { return 16 - (16 >> k); }
 
@@ -124,9 +129,8 @@ __device__ __forceinline__ unsigned row_runs(CountShared& sh, int rows, int tota
       if (d == base) prev = -16;
       sh.row[d] = (uint8_t)r;
       const int32_t after = d + 1 < total ? sh.col[0][d + 1] : INT_MAX;
-      const int32_t next = d + 1 < end ? after : INT_MAX;
-      if (c - prev >= 16) {
-        if (next - c < 16 || (CARRY && (d == base || d + 1 == end)))
+      if (apart(prev, c)) {
+        if ((d + 1 < end && !apart(c, after)) || (CARRY && (d == base || d + 1 == end)))
           runs |= 1u << (d - d0);
         else
           ++single;
@@ -186,8 +190,8 @@ __device__ __forceinline__ unsigned merge_lists(CountShared& sh, int k, int tota
         y = j < end ? src[j] : INT_MAX;
       }
       dst[d] = c;
-      if (c - prev >= 16) {
-        if (min(x, y) - c < 16 || (CARRY && (d == base || d + 1 == end)))
+      if (apart(prev, c)) {
+        if ((d + 1 < end && !apart(c, min(x, y))) || (CARRY && (d == base || d + 1 == end)))
           runs |= 1u << (d - d0);
         else
           ++single;
@@ -233,7 +237,7 @@ __device__ __forceinline__ void walk_runs(CountShared& sh, unsigned (&cnt)[4][3]
     int i = s;
     if (CARRY && s == sh.off[l << k]) {
       i = block_end<C>(col, s, stop, sh.open[0][open_base(k) + l][Q]);  // past the open block
-      if (i == stop || (i > s && col[i] - col[i - 1] >= 16)) continue;
+      if (i == stop || (i > s && apart(col[i - 1], col[i]))) continue;
     }
     unsigned n = 0;
     for (;;) {
@@ -244,7 +248,7 @@ __device__ __forceinline__ void walk_runs(CountShared& sh, unsigned (&cnt)[4][3]
         if (CARRY) sh.open[1][open_base(k) + l][Q] = first;
         break;
       }
-      if (col[i] - col[i - 1] >= 16) break;  // the next run
+      if (apart(col[i - 1], col[i])) break;  // the next run
     }
     found += (unsigned long long)n << (16 * k);
   }
