@@ -64,7 +64,7 @@ struct CountShared {
 };
 
 struct CountTask {  // one column range of a long group
-  int64_t group;
+  int64_t group;      // < 0: no range (see list_ranges)
   int32_t row, piece;  // its longest row, number of the range
 };
 
@@ -80,6 +80,27 @@ __host__ __device__ __forceinline__ int64_t pieces_of(int64_t total) { return (t
 // that the whole range [-16, 2^31) works (-16 stands before a list's first
 // column).
 __device__ __forceinline__ bool apart(int32_t a, int32_t b) { return (uint32_t)b - (uint32_t)a >= 16u; }
+
+// Lists the `np` ranges of a long group, by one warp. The list has room for
+// `cap`, which is enough for row pointers that ascend from 0 to nnz; the caller
+// may not have checked them, and pointers that fall back between two thread
+// blocks' rows hold more. A group whose ranges do not all fit is left out.
+__device__ __forceinline__ void list_ranges(CountTask* __restrict__ tasks, unsigned long long* __restrict__ ntasks,
+                                            int64_t cap, int64_t group, int longest, int64_t np) {
+  const int lane = threadIdx.x & 31;
+  unsigned long long first = 0;
+  if (lane == 0) first = atomicAdd(ntasks, (unsigned long long)np);
+  const int64_t at = (int64_t)__shfl_sync(0xffffffffu, first, 0);
+  const bool fits = at + np <= cap;
+  for (int64_t j = lane; j < np && at + j < cap; j += 32)
+    tasks[at + j] = CountTask{fits ? group : -1, longest, (int)j};
+}
+
+// the ranges that were listed
+__device__ __forceinline__ int64_t listed_ranges(const unsigned long long* __restrict__ ntasks, int64_t cap) {
+  const unsigned long long nt = *ntasks;
+  return nt < (unsigned long long)cap ? (int64_t)nt : cap;
+}
 
 // lists before level k's in CountShared::open
 __device__ __forceinline__ int open_base(int k) { return 16 - (16 >> k); }
@@ -305,13 +326,15 @@ __device__ __forceinline__ void add_counts(CountShared& sh, const unsigned (&cnt
 // most kCap entries counted, longer ones listed as tasks. acc[13] += squared
 // row lengths, acc[14] = longest row (acc[12], their sum, is nnz).
 // Rows whose pointers run backwards or leave [0, nnz] are passed over (with
-// their neighbours: the caller has not checked the CSR yet).
+// their neighbours): the caller may not have checked the CSR, and on one that is
+// not valid the three kernels stay inside their arrays and count something.
 __global__ void __launch_bounds__(kCntThreads, kCntPerSm) k_count(int64_t n, int64_t nnz,
                                                                   const int64_t* __restrict__ rowptr,
                                                                   const int32_t* __restrict__ colidx,
                                                                   unsigned long long* __restrict__ acc,
                                                                   CountTask* __restrict__ tasks,
-                                                                  unsigned long long* __restrict__ ntasks) {
+                                                                  unsigned long long* __restrict__ ntasks,
+                                                                  int64_t cap) {
   extern __shared__ __align__(16) unsigned char raw[];
   CountShared& sh = *reinterpret_cast<CountShared*>(raw);
   unsigned cnt[4][3] = {};
@@ -346,14 +369,7 @@ __global__ void __launch_bounds__(kCntThreads, kCntPerSm) k_count(int64_t n, int
             best = i;
           }
         }
-        if (threadIdx.x < 32) {
-          const int np = (int)pieces_of(own);
-          unsigned long long at = 0;
-          if (threadIdx.x == 0) at = atomicAdd(ntasks, (unsigned long long)np);
-          at = __shfl_sync(0xffffffffu, at, 0);
-          for (int j = threadIdx.x; j < np; j += 32)
-            tasks[at + j] = CountTask{row0 / 8 + g0, best, j};
-        }
+        if (threadIdx.x < 32) list_ranges(tasks, ntasks, cap, row0 / 8 + g0, best, pieces_of(own));
         ++g0;
         continue;
       }
@@ -401,14 +417,15 @@ __device__ __forceinline__ int64_t entry_from(const int32_t* __restrict__ colidx
 __global__ void __launch_bounds__(kCntThreads) k_count_cuts(int64_t n, const int64_t* __restrict__ rowptr,
                                                             const int32_t* __restrict__ colidx,
                                                             const CountTask* __restrict__ tasks,
-                                                            const unsigned long long* __restrict__ ntasks,
+                                                            const unsigned long long* __restrict__ ntasks, int64_t cap,
                                                             CountCut* __restrict__ cuts) {
   constexpr unsigned kAll = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  const int64_t nt = (int64_t)*ntasks;
+  const int64_t nt = listed_ranges(ntasks, cap);
   for (int64_t t = ((int64_t)blockIdx.x * kCntThreads + threadIdx.x) >> 5; t < nt;
        t += (int64_t)gridDim.x * (kCntThreads / 32)) {
     const CountTask tk = tasks[t];
+    if (tk.group < 0) continue;  // whole warp
     const int64_t row0 = tk.group * 8;
     const int64_t first = rowptr[row0 + tk.row], len = rowptr[row0 + tk.row + 1] - first;
     const int64_t np = pieces_of(rowptr[row0 + 8 < n ? row0 + 8 : n] - rowptr[row0]);
@@ -452,13 +469,14 @@ __global__ void __launch_bounds__(kCntThreads, kCntPerSm) k_count_long(int64_t n
                                                                        const CountTask* __restrict__ tasks,
                                                                        const CountCut* __restrict__ cuts,
                                                                        const unsigned long long* __restrict__ ntasks,
-                                                                       unsigned long long* __restrict__ acc) {
+                                                                       int64_t cap, unsigned long long* __restrict__ acc) {
   extern __shared__ __align__(16) unsigned char raw[];
   CountShared& sh = *reinterpret_cast<CountShared*>(raw);
   unsigned cnt[4][3] = {};
-  const int64_t nt = (int64_t)*ntasks;
+  const int64_t nt = listed_ranges(ntasks, cap);
   for (int64_t t = blockIdx.x; t < nt; t += gridDim.x) {
     const CountTask tk = tasks[t];
+    if (tk.group < 0) continue;  // whole block
     if (tk.piece > 0 && cuts[t].column == INT_MAX) continue;  // the range before runs on through this one
     const int64_t row0 = tk.group * 8;
     // the group's tasks follow one another
@@ -556,13 +574,13 @@ cudaError_t launch_block_counts(int64_t n, int64_t nnz, const int64_t* rowptr, c
   const int64_t pieces = (n + kCntRows - 1) / kCntRows;
   const int64_t most = (int64_t)sm_count() * kCntPerSm;
   k_count<<<(unsigned)(pieces < most ? pieces : most), kCntThreads, smem, s>>>(n, nnz, rowptr, colidx, acc, tasks,
-                                                                                  ntasks);
+                                                                                ntasks, cap);
   if (nnz > kCap) {
     const int64_t cut_blocks = (int64_t)sm_count() * 8, want = (cap * 32 + kCntThreads - 1) / kCntThreads;
     k_count_cuts<<<(unsigned)(want < cut_blocks ? want : cut_blocks), kCntThreads, 0, s>>>(n, rowptr, colidx, tasks,
-                                                                                         ntasks, cuts);
+                                                                                         ntasks, cap, cuts);
     k_count_long<<<(unsigned)(cap < most ? cap : most), kCntThreads, smem, s>>>(n, rowptr, colidx, tasks, cuts, ntasks,
-                                                                                acc);
+                                                                                cap, acc);
   }
   return cudaGetLastError();
 }

@@ -33,3 +33,26 @@ def test_columns_up_to_the_limit(cuda_device, name):
     d = spc5.upload_csr(A, torch.float64, "cuda")
     got = spc5.count_blocks(d.rowptr, d.colidx, A.n, A.m)
     assert list(got) == [oracle.beta_count(A, r, c)[1] for r, c in spc5.SHAPES]
+
+
+def still_works():
+    A = LIMIT["hub"]()
+    d = spc5.upload_csr(A, torch.float64, "cuda")
+    assert list(spc5.count_blocks(d.rowptr, d.colidx, A.n, A.m)) == [oracle.beta_count(A, r, c)[1] for r, c in spc5.SHAPES]
+
+
+def test_row_pointers_that_fall_back(cuda_device):
+    # every second 128 rows fall back to 0: the others, valid by themselves, hold four
+    # times nnz entries in long groups, more ranges than a valid CSR can have
+    nnz = 200000
+    rowptr = np.zeros(128 * 8 + 1, np.int64)
+    for piece in range(0, 8, 2):
+        rowptr[128 * piece + 1:128 * (piece + 1) + 1] = nnz
+    A = inputs.CSR(rowptr.size - 1, nnz, rowptr, np.arange(nnz, dtype=np.int32), np.ones(nnz))
+    d = spc5.upload_csr(A, torch.float32, "cuda")
+    spc5.count_blocks(d.rowptr, d.colidx, A.n, A.m)
+    spc5.features(d)
+    with pytest.raises(spc5.Spc5Error) as e:
+        spc5.tune(d)
+    assert e.value.status == spc5.EINVAL and "row 128:" in str(e.value)
+    still_works()
