@@ -486,8 +486,12 @@ __global__ void __launch_bounds__(kCntThreads, kCntPerSm) k_count_long(int64_t n
     if (threadIdx.x < 8) {
       const int64_t r = row0 + threadIdx.x;
       const int64_t a = r < n ? rowptr[r] : 0, e = r < n ? rowptr[r + 1] : 0;
-      sh.cur[threadIdx.x] = tk.piece > 0 ? cuts[t].at[threadIdx.x] : a;
-      sh.end[threadIdx.x] = next < after ? cuts[next].at[threadIdx.x] : e;
+      // both lie in the row; columns out of order can put the end before the
+      // start, and one row's negative share would hide another's length below
+      const int64_t from = tk.piece > 0 ? cuts[t].at[threadIdx.x] : a;
+      const int64_t to = next < after ? cuts[next].at[threadIdx.x] : e;
+      sh.cur[threadIdx.x] = from;
+      sh.end[threadIdx.x] = to > from ? to : from;
     }
     if (threadIdx.x < kLists * 3) sh.open[0][threadIdx.x / 3][threadIdx.x % 3] = -16;
     for (;;) {

@@ -56,3 +56,19 @@ def test_row_pointers_that_fall_back(cuda_device):
         spc5.tune(d)
     assert e.value.status == spc5.EINVAL and "row 128:" in str(e.value)
     still_works()
+
+
+def test_hubs_with_columns_out_of_order(cuda_device):
+    # the cuts of such a group do not ascend: a range can end before it starts in one row
+    # and hold thousands of entries in another
+    rng = np.random.default_rng(0)
+    rows = [rng.permutation(2_000_000)[:k] for k in (30000, 30000, 5, 2, 20000, 3, 9, 1)]
+    rows += [rng.permutation(50_000)[:k] for k in (9, 0, 7000, 6000, 5000, 4000, 3000, 2500)]
+    A = csr(rows + [np.arange(40)] * 5, 2_000_000)
+    d = spc5.upload_csr(A, torch.float32, "cuda")
+    spc5.count_blocks(d.rowptr, d.colidx, A.n, A.m)
+    spc5.features(d)
+    with pytest.raises(spc5.Spc5Error) as e:
+        spc5.tune(d)
+    assert e.value.status == spc5.EUNSORTED and "row 0:" in str(e.value)
+    still_works()
