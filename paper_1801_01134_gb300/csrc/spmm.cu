@@ -608,14 +608,15 @@ __global__ void __launch_bounds__(128) k_spmm_seg4(int64_t nseg, const Segment* 
   const typename T::V* __restrict__ v = val + sg.v_begin;
   const float* __restrict__ xj = X + (own ? j : 0);
   float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int32_t b0 = sg.b_begin; b0 < sg.b_end; b0 += 2 * kWarp) {
+  const uint32_t end = (uint32_t)sg.b_end;  // unsigned: a trip may pass 2^31 - 1 where the last blocks lie there
+  for (uint32_t b0 = (uint32_t)sg.b_begin; b0 < end; b0 += 2 * kWarp) {
     uint32_t m[2], at[2];
     int first[2], sum = 0;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const int32_t b = b0 + h * kWarp + lane;
-      m[h] = b < sg.b_end ? load_mask<MB>(bmask, b).w[0] : 0u;
-      at[h] = b < sg.b_end ? (uint32_t)__ldg(bcol + b) * ldx : 0u;
+      const uint32_t b = b0 + h * kWarp + lane;
+      m[h] = b < end ? load_mask<MB>(bmask, b).w[0] : 0u;
+      at[h] = b < end ? (uint32_t)__ldg(bcol + b) * ldx : 0u;
     }
 #pragma unroll
     for (int h = 0; h < 2; ++h) {

@@ -763,18 +763,20 @@ __device__ __forceinline__ typename T::A segment_sum_r1(const Segment& sg, const
   const int lane = threadIdx.x & 31;
   const typename T::V* __restrict__ v = val + sg.v_begin;
   A acc0 = 0, acc1 = 0;
-  int32_t b = sg.b_begin + lane;
-  uint32_t n0 = b < sg.b_end ? load_mask<MB>(bmask, b).w[0] : 0u;
-  uint32_t n1 = b + 32 < sg.b_end ? load_mask<MB>(bmask, b + 32).w[0] : 0u;
-  int32_t d0 = b < sg.b_end ? __ldg(bcol + b) : 0, d1 = b + 32 < sg.b_end ? __ldg(bcol + b + 32) : 0;
-  for (int32_t t = sg.b_begin; t < sg.b_end; t += 64) {
+  // unsigned: the look ahead may pass 2^31 - 1 where the last blocks lie there
+  const uint32_t end = (uint32_t)sg.b_end;
+  uint32_t b = (uint32_t)sg.b_begin + lane;
+  uint32_t n0 = b < end ? load_mask<MB>(bmask, b).w[0] : 0u;
+  uint32_t n1 = b + 32 < end ? load_mask<MB>(bmask, b + 32).w[0] : 0u;
+  int32_t d0 = b < end ? __ldg(bcol + b) : 0, d1 = b + 32 < end ? __ldg(bcol + b + 32) : 0;
+  for (uint32_t t = (uint32_t)sg.b_begin; t < end; t += 64) {
     uint32_t m0 = n0, m1 = n1;
     const int32_t c0 = d0, c1 = d1;
     b += 64;  // the next trip's blocks
-    n0 = b < sg.b_end ? load_mask<MB>(bmask, b).w[0] : 0u;
-    n1 = b + 32 < sg.b_end ? load_mask<MB>(bmask, b + 32).w[0] : 0u;
-    d0 = b < sg.b_end ? __ldg(bcol + b) : 0;
-    d1 = b + 32 < sg.b_end ? __ldg(bcol + b + 32) : 0;
+    n0 = b < end ? load_mask<MB>(bmask, b).w[0] : 0u;
+    n1 = b + 32 < end ? load_mask<MB>(bmask, b + 32).w[0] : 0u;
+    d0 = b < end ? __ldg(bcol + b) : 0;
+    d1 = b + 32 < end ? __ldg(bcol + b + 32) : 0;
     const int own = __popc(m0) | (__popc(m1) << 16);
     int incl = own;
 #pragma unroll
