@@ -296,7 +296,7 @@ __global__ void k_r1_fill(int64_t n, int64_t nnz, int c, int mb, int seg_blocks,
 }
 
 // ------------------------------------------------------ tiles of intervals
-// r > 1: a thread block takes kTileIntervals intervals and brings the columns
+// r > 1: a thread block takes up to kTileIntervals intervals and brings the columns
 // of as many as fit (kTileEntries entries at a time) into shared memory with
 // consecutive reads; one lane per row then walks the merged cover there. Walking the rows in global memory waited for it at every step (27-
 // point stencil 128^3, beta(4,8): 0.18 ms to count, 0.36 to fill, then 0.41 to
@@ -308,11 +308,23 @@ __global__ void k_r1_fill(int64_t n, int64_t nnz, int c, int mb, int seg_blocks,
 // DRAM: columns read twice, values read and written once. Measured for that
 // matrix (float64, n = 2.1 M, 56 M entries): check and count 0.12 ms, fill and
 // values 0.29; the whole conversion 1.22 -> 0.58 ms.
-// Intervals with more than kTileEntries entries go to a list for the kernels
+// Intervals with more than kListEntries entries go to a list for the kernels
 // that walk global memory.
 constexpr int kTileThreads = 256;
-constexpr int kTileIntervals = 64;
 constexpr int kTileEntries = 4096;
+// Intervals of a thread block, at most. At R = 2, 64 left half of the lanes idle
+// (one million rows of 8 scattered entries, beta(2,4): 0.51 ms; 128, and one
+// shuffle per block of the cover instead of three, 0.38).
+template <int R>
+constexpr int kTileIntervals = R == 2 ? 128 : 64;
+// An interval with more entries is listed. Few of them fit a tile, so a block
+// walks them with most of its lanes idle and one step after another, where the
+// list has a warp for each. Measured against one limit of 4096, float64: R-MAT
+// scale 16, beta(4,4), 6.9 -> 3.75 ms; 40 thousand rows of 300 entries, beta(2,4),
+// 4.3 -> 1.5. At R = 8 a band of 520 entries an interval takes 0.33 ms in the
+// tiles and 0.63 in the list, so the line lies higher there.
+template <int R>
+constexpr int kListEntries = R == 8 ? 1024 : 512;
 
 struct TileList {  // device: intervals too long for a tile
   unsigned long long count;
@@ -354,13 +366,34 @@ __device__ __forceinline__ int32_t cover_tile(const int32_t* __restrict__ col, i
   return nb;
 }
 
+// Which of the intervals [a, b) a thread walks with its R lanes: the first, and
+// the distance to its next one. Neighbouring lanes take neighbouring intervals;
+// where there is a warp for every interval each has its own, since those of one
+// warp take turns.
+template <int R>
+__device__ __forceinline__ int tile_interval(int a, int b, int* step) {
+  *step = kTileThreads / R;
+  if (b - a > kTileThreads / kWarp) return a + (int)threadIdx.x / R;
+  return (threadIdx.x & 31) < R ? a + (int)(threadIdx.x >> 5) : b;
+}
+
 // The intervals [a, b) of the tile whose rows start at rel[], as many from a
-// on as fit; rel holds kTileIntervals * R + 1 row starts.
+// on as fit and are not for the list, or the one at a that is (tile_listed); rel
+// holds kTileIntervals<R> * R + 1 row starts. Every warp looks for itself.
 template <int R>
 __device__ __forceinline__ int tile_step(const int32_t* rel, int a, int intervals) {
-  int b = a + 1;
-  while (b < intervals && rel[(b + 1) * R] - rel[a * R] <= kTileEntries) ++b;
-  return b;
+  if (rel[(a + 1) * R] - rel[a * R] > kListEntries<R>) return a + 1;
+  for (int b = a + 1;; b += kWarp) {
+    const int k = b + (threadIdx.x & 31);
+    const bool stop = k >= intervals || rel[(k + 1) * R] - rel[a * R] > kTileEntries ||
+                      rel[(k + 1) * R] - rel[k * R] > kListEntries<R>;
+    const unsigned who = __ballot_sync(0xffffffffu, stop);
+    if (who) return b + __ffs(who) - 1;
+  }
+}
+template <int R>
+__device__ __forceinline__ bool tile_listed(int a, int b, int total) {
+  return b == a + 1 && total > kListEntries<R>;
 }
 
 // CSR check and block counts. *status = 0 when anything is wrong (the
@@ -372,15 +405,15 @@ __global__ void __launch_bounds__(kTileThreads) k_tile_count(int64_t n, int64_t 
                                                              int32_t* __restrict__ counts,
                                                              unsigned long long* __restrict__ status,
                                                              TileList* __restrict__ list, int64_t* __restrict__ longs,
-                                                             int64_t cap) {
-  constexpr int kRows = kTileIntervals * R;
+                                                             int64_t cap, int per_block) {
+  const int kRows = per_block * R;
   __shared__ int32_t col[kTileEntries];
-  __shared__ int32_t rel[kRows + 1];
+  __shared__ int32_t rel[kTileIntervals<R> * R + 1];
   const int tid = threadIdx.x;
   const unsigned group = ((1u << R) - 1u) << (tid & 31 & ~(R - 1));  // the lanes of an interval
-  const int64_t it0 = (int64_t)blockIdx.x * kTileIntervals;
+  const int64_t it0 = (int64_t)blockIdx.x * per_block;
   const int64_t row0 = it0 * R;
-  const int intervals = I - it0 < kTileIntervals ? (int)(I - it0) : kTileIntervals;
+  const int intervals = I - it0 < per_block ? (int)(I - it0) : per_block;
   const int64_t base = rowptr[row0];
   bool bad = row0 == 0 && base != 0;
   for (int r = tid; r <= kRows; r += kTileThreads) {
@@ -396,7 +429,7 @@ __global__ void __launch_bounds__(kTileThreads) k_tile_count(int64_t n, int64_t 
   for (int a = 0; a < intervals;) {
     const int b = tile_step<R>(rel, a, intervals);
     const int start = rel[a * R], total = rel[b * R] - start;
-    if (total > kTileEntries) {  // one long interval: checked here, counted from the list
+    if (tile_listed<R>(a, b, total)) {  // one long interval: checked here, counted from the list
       for (int r = a * R; r < b * R; ++r)
         for (int64_t p = base + rel[r] + tid; p < base + rel[r + 1]; p += kTileThreads) {
           const int32_t v = colidx[p];
@@ -412,7 +445,8 @@ __global__ void __launch_bounds__(kTileThreads) k_tile_count(int64_t n, int64_t 
 #pragma unroll 4
     for (int s = tid; s < total; s += kTileThreads) col[s] = __ldg(colidx + base + start + s);
     __syncthreads();
-    for (int it = a + tid / R; it < b; it += kTileThreads / R) {
+    int step;
+    for (int it = tile_interval<R>(a, b, &step); it < b; it += step) {
       const int r = it * R + tid % R;
       const int32_t nb = cover_tile<R, true>(col, rel[r] - start, rel[r + 1] - start, c, group, m, &bad,
                                              [](int32_t, int, int, uint32_t) {});
@@ -477,8 +511,8 @@ struct BlockSink {
 };
 
 template <int R>
-__device__ __forceinline__ void write_block(const BlockSink& out, int i, int c, unsigned group, int32_t blk, int32_t s,
-                                            uint32_t bits, int64_t v) {
+__device__ __forceinline__ void write_block(const BlockSink& out, int i, int c, int32_t blk, int32_t s, uint32_t bits,
+                                            uint32_t next, int64_t v) {
   if (i == 0) {
     out.bcol[blk] = s;
     const int32_t jb = blk - out.b0;
@@ -494,7 +528,6 @@ __device__ __forceinline__ void write_block(const BlockSink& out, int i, int c, 
   }
   // every lane writes its row's mask bits; two rows of 4 share a byte
   if (c == 4) {
-    const uint32_t next = __shfl_down_sync(group, bits, 1, R);
     if (!(i & 1)) out.bmask[(int64_t)blk * (R / 2) + i / 2] = (uint8_t)(bits | (next << 4));
   } else if (c == 8) {
     out.bmask[(int64_t)blk * R + i] = (uint8_t)bits;
@@ -503,9 +536,17 @@ __device__ __forceinline__ void write_block(const BlockSink& out, int i, int c, 
   }
 }
 
-// exclusive sum over the R lanes of an interval; *total the sum
+// entries of a block in the rows before lane i's, from the rows' bits; *total in
+// all of them, *next the next lane's bits (for c = 4, where two rows share a byte)
 template <int R>
-__device__ __forceinline__ int lanes_before(int v, int i, unsigned group, int* total) {
+__device__ __forceinline__ int lanes_before(uint32_t bits, int i, int c, unsigned group, int* total, uint32_t* next) {
+  const int v = __popc(bits);
+  if constexpr (R == 2) {
+    *next = __shfl_xor_sync(group, bits, 1, R);
+    *total = v + __popc(*next);
+    return i == 0 ? 0 : *total - v;
+  }
+  *next = c == 4 ? __shfl_down_sync(group, bits, 1, R) : 0u;
   int in = v;
 #pragma unroll
   for (int d = 1; d < R; d <<= 1) {
@@ -525,30 +566,32 @@ __global__ void __launch_bounds__(kTileThreads) k_tile_fill(int64_t n, int64_t I
                                                             const int32_t* __restrict__ brp,
                                                             const int32_t* __restrict__ segptr,
                                                             int32_t* __restrict__ bcol, uint8_t* __restrict__ bmask,
-                                                            VT* __restrict__ bval, Segment* __restrict__ segs) {
-  constexpr int kRows = kTileIntervals * R;
+                                                            VT* __restrict__ bval, Segment* __restrict__ segs,
+                                                            int per_block) {
+  const int kRows = per_block * R;
   __shared__ int32_t col[kTileEntries];
-  __shared__ int32_t rel[kRows + 1];
+  __shared__ int32_t rel[kTileIntervals<R> * R + 1];
   __shared__ uint16_t from[kTileEntries];  // CSR place of the value at each place in block order
   const int tid = threadIdx.x;
   const unsigned group = ((1u << R) - 1u) << (tid & 31 & ~(R - 1));  // the lanes of an interval
-  const int64_t it0 = (int64_t)blockIdx.x * kTileIntervals;
+  const int64_t it0 = (int64_t)blockIdx.x * per_block;
   const int64_t row0 = it0 * R;
-  const int intervals = I - it0 < kTileIntervals ? (int)(I - it0) : kTileIntervals;
+  const int intervals = I - it0 < per_block ? (int)(I - it0) : per_block;
   const int64_t base = rowptr[row0];
   for (int r = tid; r <= kRows; r += kTileThreads) rel[r] = (int32_t)(rowptr[row0 + r < n ? row0 + r : n] - base);
   __syncthreads();
   for (int a = 0; a < intervals;) {
     const int b = tile_step<R>(rel, a, intervals);
     const int start = rel[a * R], total = rel[b * R] - start;
-    if (total > kTileEntries) {
+    if (tile_listed<R>(a, b, total)) {
       a = b;
       continue;
     }
 #pragma unroll 4
     for (int s = tid; s < total; s += kTileThreads) col[s] = __ldg(colidx + base + start + s);
     __syncthreads();
-    for (int it = a + tid / R; it < b; it += kTileThreads / R) {
+    int step;
+    for (int it = tile_interval<R>(a, b, &step); it < b; it += step) {
       const int i = tid % R, r = it * R + i;
       const int32_t b0 = brp[it0 + it];
       const bool is_long = segptr != nullptr && segptr[it0 + it + 1] > segptr[it0 + it];
@@ -558,9 +601,10 @@ __global__ void __launch_bounds__(kTileThreads) k_tile_fill(int64_t n, int64_t I
       int to = rel[it * R] - start;  // place in block order of the block's first value
       cover_tile<R, false>(col, rel[r] - start, rel[r + 1] - start, c, group, 0, nullptr,
                            [&](int32_t s, int h0, int h1, uint32_t bits) {
-                             write_block<R>(out, i, c, group, blk, s, bits, base + start + to);
                              int all;
-                             int q = to + lanes_before<R>(h1 - h0, i, group, &all);
+                             uint32_t next;
+                             int q = to + lanes_before<R>(bits, i, c, group, &all, &next);
+                             write_block<R>(out, i, c, blk, s, bits, next, base + start + to);
                              for (int p = h0; p < h1; ++p, ++q) from[q] = (uint16_t)p;
                              to += all;
                              ++blk;
@@ -598,10 +642,11 @@ __global__ void __launch_bounds__(64) k_fill(int64_t n, int64_t nlist, const int
   int64_t v = 0;
   cover_tile<R, false>(colidx + base, (int)(a - base), (int)(e - base), c, group, 0, nullptr,
                        [&](int32_t s, int h0, int h1, uint32_t bits) {
-                         write_block<R>(out, i, c, group, blk, s, bits, base + v);
-                         if (i == 0) bvo[blk] = (int32_t)v;
                          int total;
-                         lanes_before<R>(h1 - h0, i, group, &total);
+                         uint32_t next;
+                         lanes_before<R>(bits, i, c, group, &total, &next);
+                         write_block<R>(out, i, c, blk, s, bits, next, base + v);
+                         if (i == 0) bvo[blk] = (int32_t)v;
                          v += total;
                          ++blk;
                        });
@@ -862,14 +907,27 @@ spc5_status scan_counts(const int32_t* in, int64_t L, int32_t* out, int64_t* tot
   return SPC5_OK;
 }
 
+// Intervals of one thread block: where the most allowed would take more than two
+// steps, as many as fill a tile on average, so that blocks of longer rows do not
+// walk them a few at a time, one step after another, while others of the GPU's
+// SMs have none (banded, 520 entries an interval, beta(8,4): 0.50 -> 0.33 ms).
+template <int R>
+int tile_intervals(int64_t nnz, int64_t I) {
+  const int64_t mean = nnz / (I > 0 ? I : 1) + 1;
+  const int64_t per = kTileEntries / mean;
+  return (int)(per < 1 ? 1 : per > kTileIntervals<R> / 2 ? kTileIntervals<R> : per);
+}
+
 // r > 1: CSR check and block counts (see k_tile_count)
 template <int R>
 void launch_tile_count(int64_t n, int64_t m, int64_t nnz, int64_t I, int c, const int64_t* rowptr,
                        const int32_t* colidx, int32_t* counts, unsigned long long* status, TileList* list,
                        int64_t* longs, cudaStream_t s) {
-  const unsigned grid = (unsigned)((I + kTileIntervals - 1) / kTileIntervals);
-  const int64_t cap = nnz / kTileEntries;  // at most so many intervals are listed
-  k_tile_count<R><<<grid, kTileThreads, 0, s>>>(n, m, nnz, I, c, rowptr, colidx, counts, status, list, longs, cap);
+  const int per_block = tile_intervals<R>(nnz, I);
+  const unsigned grid = (unsigned)((I + per_block - 1) / per_block);
+  const int64_t cap = nnz / kListEntries<R>;  // at most so many intervals are listed
+  k_tile_count<R><<<grid, kTileThreads, 0, s>>>(n, m, nnz, I, c, rowptr, colidx, counts, status, list, longs, cap,
+                                             per_block);
   if (cap > 0) k_count<R><<<(unsigned)((cap + 1) / 2), 64, 0, s>>>(n, c, rowptr, colidx, list, longs, cap, counts);
 }
 
@@ -877,11 +935,12 @@ template <int R, class VT>
 void launch_tile_fill(int64_t n, int64_t I, int c, int mb, int sb, const int64_t* rowptr, const int32_t* colidx,
                       const void* values, const int32_t* segptr, int64_t nlist, const int64_t* longs, int32_t* bvo,
                       spc5_matrix* h, cudaStream_t s) {
-  const unsigned grid = (unsigned)((I + kTileIntervals - 1) / kTileIntervals);
+  const int per_block = tile_intervals<R>(h->nnz, I);
+  const unsigned grid = (unsigned)((I + per_block - 1) / per_block);
   const VT* v = (const VT*)values;
   VT* bv = (VT*)h->values;
   k_tile_fill<R, VT><<<grid, kTileThreads, 0, s>>>(n, I, c, sb, rowptr, colidx, v, h->block_rowptr, segptr,
-                                                   h->block_colidx, h->block_masks, bv, h->segs);
+                                                   h->block_colidx, h->block_masks, bv, h->segs, per_block);
   if (nlist > 0) {
     k_fill<R><<<(unsigned)((nlist + 1) / 2), 64, 0, s>>>(n, nlist, longs, c, sb, rowptr, colidx, h->block_rowptr,
                                                           segptr, h->block_colidx, h->block_masks, bvo, h->segs);
@@ -1539,7 +1598,7 @@ spc5_status convert_impl(int64_t n, int64_t m, int64_t nnz, const int64_t* rowpt
   int64_t* longs = nullptr;
   TileList listed{0, 0};
   if (n > 0 && r > 1) {
-    e = list.alloc(sizeof(TileList) + sizeof(int64_t) * (size_t)(nnz / kTileEntries + 1), s);
+    e = list.alloc(sizeof(TileList) + sizeof(int64_t) * (size_t)(nnz / kListEntries<2> + 1), s);  // the smallest limit
     if (e == cudaSuccess) e = cudaMemsetAsync(list.p, 0, sizeof(TileList), s);
     if (e != cudaSuccess) return bail(cuda_fail(e, "convert: interval list"));
     TileList* head = (TileList*)list.p;
