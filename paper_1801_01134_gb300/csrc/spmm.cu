@@ -276,8 +276,9 @@ __device__ __forceinline__ float4 load_x4(const float* __restrict__ X, uint32_t 
 // and Y, k and the leading dimensions multiples of 4) and 32 bits address X:
 // the same mapping and the same sums. The general kernel spends about thirty
 // instructions per stored value on bit searches, 64-bit address products and
-// the tests of a partial slice; here they are about half. With c = 4 the bit
-// positions are unrolled, so a block's X slices are all on the way at once.
+// the tests of a partial slice; here they are about half. With FULL (c = 4,
+// blocks of two and more values) the bit positions are unrolled, so a block's X
+// slices are all on the way at once.
 // With ORDER the intervals come in the handle's sorted work order (intervals
 // of similar length share a warp).
 // With r > 1 a column's X slice is read once for all the rows that hold it,
@@ -286,10 +287,11 @@ __device__ __forceinline__ float4 load_x4(const float* __restrict__ X, uint32_t 
 // 128^3, k = 32, beta(1,4) 0.557 -> 0.466 ms, beta(2,4) 0.568 -> 0.376 (four
 // rows per block 0.482: more tests than reads saved); R-MAT scale 22, k = 8,
 // the short rows 0.54 -> 0.47 ms in natural order and about 0.22 in the sorted
-// one. Unrolling beta(1,4) is worth 15 % where blocks hold three values (FEM)
-// and costs 40 % where they hold one (R-MAT; beta(1,8) keeps the bit loop, and
-// the tuner picks).
-template <class T, int R, int C, int G, bool ORDER>
+// one. FULL has its line at two values per block: beta(1,4), k = 32, unrolled, bit
+// by bit and in the general kernel, 7-point 100^3 (1.4 values) 0.178, 0.130 and
+// 0.144 ms, uniform 500 thousand rows (1.0) 0.136, 0.096, 0.104; with three
+// values (27-point 64^3, FEM) unrolled is 1.2 and 1.4 times the general kernel.
+template <class T, int R, int C, int G, bool ORDER, bool FULL>
 __global__ void __launch_bounds__(256) k_spmm_blk4(int64_t n, int64_t I, int32_t long_blocks, int64_t long_values,
                                                    const int32_t* __restrict__ brp, const int32_t* __restrict__ bcol,
                                                    const uint8_t* __restrict__ bmask,
@@ -322,7 +324,7 @@ __global__ void __launch_bounds__(256) k_spmm_blk4(int64_t n, int64_t I, int32_t
       m0 = load_mask<MB>(bmask, b + 1);
       c0 = (uint32_t)__ldg(bcol + b + 1);
     }
-    if constexpr (R == 1 && C == 4) {
+    if constexpr (R == 1 && FULL) {
       const uint32_t bits = mk.w[0];
       float vv[4];
       float4 xx[4];
@@ -352,7 +354,7 @@ __global__ void __launch_bounds__(256) k_spmm_blk4(int64_t n, int64_t I, int32_t
         vo[i] = popc_below<C>(mk, i);
         uni |= rb[i];
       }
-      if constexpr (C == 4) {
+      if constexpr (FULL) {
         float4 xx[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q)
@@ -390,7 +392,16 @@ void launch_spmm_blk(const spc5_matrix* h, int k, const typename T::X* Xm, int64
   // 16-byte X loads when every lane's 4 columns start on a 16-byte boundary
   const bool vec = sizeof(typename T::X) == 4 && ldx % 4 == 0 && (reinterpret_cast<uintptr_t>(Xm) & 15u) == 0;
   if constexpr (sizeof(typename T::X) == 4) {
-    if (vec && k % 4 == 0 && ldy % 4 == 0 && (reinterpret_cast<uintptr_t>(Ym) & 15u) == 0 && h->m * ldx < (int64_t)INT32_MAX) {
+    // Blocks of eight rows and eight or sixteen columns that are neither nearly
+    // empty nor half full: a column is tested against eight rows, of which one
+    // to three hold it on a grid. With four and more lanes to an interval the
+    // general kernel, which walks value by value, is ahead there: 7-point 100^3,
+    // beta(8,8), k = 32, 0.156 against 0.209 ms, 27-point 64^3 0.117 against
+    // 0.134 (FEM with three equal rows to a block row 0.74 against 0.52: no count
+    // that the handle has tells the two apart).
+    const bool shared = h->r < 8 || h->c < 8 || G < 4 || h->nnz < 2 * h->nb || 2 * h->nnz >= (int64_t)h->r * h->c * h->nb;
+    if (shared && vec && k % 4 == 0 && ldy % 4 == 0 && (reinterpret_cast<uintptr_t>(Ym) & 15u) == 0 &&
+        h->m * ldx < (int64_t)INT32_MAX) {
       const bool ordered = ordered_variant(h->variant) && h->norder > 0;
       const int64_t slots = ordered ? h->norder : h->I;
       const dim3 g4((unsigned)((slots * G + 255) / 256), grid.y);
@@ -398,12 +409,16 @@ void launch_spmm_blk(const spc5_matrix* h, int k, const typename T::X* Xm, int64
         kern<<<g4, 256, 0, s>>>(h->n, h->I, h->long_blocks, h->long_values, h->block_rowptr, h->block_colidx,
                                 h->block_masks, val, h->valptr, Xm, (uint32_t)ldx, Ym, ldy, k, h->order, h->norder);
       };
-#define SPC5_BLK4(RR, CC) \
-  if (h->r == RR && h->c == CC) return ordered ? go(k_spmm_blk4<T, RR, CC, G, true>) : go(k_spmm_blk4<T, RR, CC, G, false>);
-      SPC5_BLK4(1, 4) SPC5_BLK4(1, 8) SPC5_BLK4(1, 16)
-      SPC5_BLK4(2, 4) SPC5_BLK4(2, 8) SPC5_BLK4(2, 16)
-      SPC5_BLK4(4, 4) SPC5_BLK4(4, 8) SPC5_BLK4(4, 16)
-      SPC5_BLK4(8, 4) SPC5_BLK4(8, 8) SPC5_BLK4(8, 16)
+#define SPC5_BLK4(RR, CC, FULL)   \
+  if (h->r == RR && h->c == CC) \
+    return ordered ? go(k_spmm_blk4<T, RR, CC, G, true, FULL>) : go(k_spmm_blk4<T, RR, CC, G, false, FULL>);
+      if (h->nnz >= 2 * h->nb) {
+        SPC5_BLK4(1, 4, true) SPC5_BLK4(2, 4, true) SPC5_BLK4(4, 4, true) SPC5_BLK4(8, 4, true)
+      }
+      SPC5_BLK4(1, 4, false) SPC5_BLK4(1, 8, false) SPC5_BLK4(1, 16, false)
+      SPC5_BLK4(2, 4, false) SPC5_BLK4(2, 8, false) SPC5_BLK4(2, 16, false)
+      SPC5_BLK4(4, 4, false) SPC5_BLK4(4, 8, false) SPC5_BLK4(4, 16, false)
+      SPC5_BLK4(8, 4, false) SPC5_BLK4(8, 8, false) SPC5_BLK4(8, 16, false)
 #undef SPC5_BLK4
     }
   }
