@@ -509,7 +509,9 @@ __device__ __forceinline__ bool grid_sum(A mine, ResState* st, unsigned phase, T
 
 // acc = row `row` of A times x, its `len` entries from col and val (stride 32)
 // on, eight (float64: four, for the registers) at a time: their loads are all
-// on the way before the first is used.
+// on the way before the first is used. Values stay as they are stored until
+// then: widening bfloat16 at the load made every load wait for the one before
+// (27-point 96^3, beta(2,4), an iteration 85 us; now 47, float32 52).
 // x changes while the kernel runs: ordinary loads, not read-only ones.
 template <class T>
 __device__ __forceinline__ typename T::A row_dot(int len, const int32_t* __restrict__ col,
@@ -518,19 +520,20 @@ __device__ __forceinline__ typename T::A row_dot(int len, const int32_t* __restr
   typename T::A acc = 0;
   for (int j = 0; j < len; j += U) {
     int32_t c[U];
-    typename T::A v[U], xx[U];
+    typename T::V v[U];
+    typename T::A xx[U];
 #pragma unroll
     for (int u = 0; u < U; ++u)
       if (j + u < len) {
         c[u] = __ldg(col + 32 * (j + u));
-        v[u] = T::val(val, 32 * (j + u));
+        v[u] = __ldg(val + 32 * (j + u));
       }
 #pragma unroll
     for (int u = 0; u < U; ++u)
       if (j + u < len) xx[u] = x[c[u]];
 #pragma unroll
     for (int u = 0; u < U; ++u)
-      if (j + u < len) acc = fmadd<T>(v[u], xx[u], acc);
+      if (j + u < len) acc = fmadd<T>(sval<T>(v, u), xx[u], acc);
   }
   return acc;
 }
