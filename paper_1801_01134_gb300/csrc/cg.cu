@@ -30,6 +30,7 @@
 // replayed, and the host reads the residual norm every `check_every`
 // iterations.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <vector>
 
@@ -335,6 +336,19 @@ __global__ void __launch_bounds__(kThreads) k_cg_xr_fused(T* __restrict__ x, T* 
 constexpr int kResThreads = 512;
 constexpr int kResPerSm = 2;
 constexpr size_t kResReserve = 16384;  // shared memory left to the block's own words and the system
+// Rows of a thread held in shared memory, at most. The L1 takes what they leave,
+// and a float64 product that gathers all over r needs room there for its loads
+// on the way: two million rows of 8 scattered entries, an iteration 208 us with
+// the seven rows that fit, 122 with five, 118 with four; 7-point 128^3 98.7, 102
+// and 104 (float32 there 45, and 53 with half of its rows).
+template <class X>
+constexpr int kResHeld = sizeof(X) == 8 ? 5 : INT_MAX;
+// A float64 thread with more rows than this many times those it holds streams
+// its vectors through the L2 like the separate kernels do, with half their
+// threads on the way: 7-point 160^3 (4.1 million rows, 27 of them per thread)
+// 185 us an iteration against 174 to 178, 128^3 (14 per thread) 102 against 101.
+// In float32 the resident kernel stays ahead (200^3: 198 against 248 us).
+constexpr int kResStream = 4;
 constexpr long long kSpinClocks = 4000000000ll;  // about two seconds
 
 // Unpacked rows of a matrix (device), 32 rows per slice.
@@ -697,7 +711,9 @@ ResLaunch resident_kernel(int64_t n) {
   const int64_t blocks = std::min({(n + kResThreads - 1) / kResThreads, (int64_t)sm_count() * per_sm, (int64_t)kResThreads});
   const size_t row = 3 * sizeof(typename T::X) * kResThreads;  // one row of every thread
   const size_t room = std::min((size_t)smem_block, (size_t)smem_sm / (size_t)per_sm) - kResReserve;
-  l.held = (int)std::min((n + blocks * kResThreads - 1) / (blocks * kResThreads), (int64_t)(room / row));
+  const int64_t each = (n + blocks * kResThreads - 1) / (blocks * kResThreads);  // rows of a thread
+  l.held = (int)std::min({each, (int64_t)(room / row), (int64_t)kResHeld<typename T::X>});
+  if (sizeof(typename T::X) == 8 && each > kResStream * (int64_t)l.held) return l;
   l.smem = row * (size_t)l.held;
   int fit = 0;
   if (cudaFuncSetAttribute(l.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room) == cudaSuccess &&

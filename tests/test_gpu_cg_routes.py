@@ -41,3 +41,37 @@ def test_bfloat16_rows_cost_no_more_than_float32(cuda_device):
     run = {t: seconds(lambda: spc5.cg(M, b, A_inner=L, tol=1e-25, max_iters=200, reliable=True))
            for t in (torch.float32, torch.bfloat16) for L in [convert(A, t, 2, 4)]}
     assert run[torch.bfloat16] <= 1.25 * run[torch.float32]
+
+
+def scattered(n, per):
+    """n rows of `per` entries spread over all columns, the diagonal among them (on the GPU)."""
+    g = torch.Generator("cuda").manual_seed(n)
+    cols = torch.randint(0, n // per, (n, per), generator=g, device="cuda") + torch.arange(per, device="cuda") * (n // per)
+    i = torch.arange(n, device="cuda")
+    cols[i, (i // (n // per)).clamp(max=per - 1)] = i
+    cols = cols.sort(1).values
+    vals = torch.where(cols == i[:, None], per - 1.0 + 1e-4, -1.0).double()
+    return torch.arange(n + 1, device="cuda") * per, cols.int().reshape(-1), vals.reshape(-1)
+
+
+def test_scattered_float64_rows_keep_their_loads_on_the_way(cuda_device):
+    n = 2000000
+    rowptr, cols, vals = scattered(n, 8)
+    M = spc5.convert(rowptr, cols, vals, n, n, 1, 4)
+    L = spc5.convert(rowptr, cols, vals.float(), n, n, 1, 4)
+    b = torch.rand(n, dtype=torch.float64, device="cuda")
+    # an iteration: float32 98 us, float64 122 (208 where its rows left the L1 no room)
+    f64 = seconds(lambda: spc5.cg(M, b, tol=1e-25, max_iters=200))
+    f32 = seconds(lambda: spc5.cg(M, b, A_inner=L, tol=1e-25, max_iters=200, reliable=True))
+    assert f64 <= 1.6 * f32
+
+
+@pytest.mark.parametrize("nz", [138, 139])  # 3,105,000 and 3,127,500 rows: either side of twenty rows per thread
+def test_float64_rows_around_the_change_of_route(cuda_device, nz):
+    A = inputs.poisson_shifted(150, 150, nz, seed=4)
+    M = convert(A, torch.float64, 1, 4)
+    b = torch.from_numpy(inputs.vec_uniform(A.n, seed=1)).cuda()
+    x, info = spc5.cg(M, b, tol=1e-10)
+    assert info["converged"] and info["rel_residual"] <= 1e-10
+    y, again = spc5.cg(M, b, tol=1e-10, use_graph=True)
+    assert again == info and torch.equal(x, y)
