@@ -502,7 +502,11 @@ typedef struct {
                               reliable updates (the float64 residual replaces
                               the recurred one whenever its norm fell 10x; no
                               restarts) instead of refinement   [0: refinement] */
-  int32_t reserved[4];
+  int32_t wait_us;         /* longest wait of the resident kernel's thread blocks
+                              for one another, about; a solve in which one waits
+                              longer is done again with separate kernels
+                              [0: two seconds] */
+  int32_t reserved[3];
 } spc5_cg_opts;
 
 typedef struct {

@@ -332,7 +332,9 @@ __global__ void __launch_bounds__(kThreads) k_cg_xr_fused(T* __restrict__ x, T* 
 // the product (blocks finish unevenly), 1.3 the updates, 3 and 6 the two
 // barriers (the second waits until the new r can be read everywhere); float64
 // spends 19 us on its pipe's multiply-adds alone.
-// Waits are bounded: a block that gives up sets the status and all leave.
+// Waits are bounded: a block that gives up sets the status and all leave. The
+// solve is then done again with the separate kernels, and so is one whose launch
+// is refused (a context that owns fewer SMs than the device has).
 constexpr int kResThreads = 512;
 constexpr int kResPerSm = 2;
 constexpr size_t kResReserve = 16384;  // shared memory left to the block's own words and the system
@@ -349,7 +351,7 @@ constexpr int kResHeld = sizeof(X) == 8 ? 5 : INT_MAX;
 // 185 us an iteration against 174 to 178, 128^3 (14 per thread) 102 against 101.
 // In float32 the resident kernel stays ahead (200^3: 198 against 248 us).
 constexpr int kResStream = 4;
-constexpr long long kSpinClocks = 4000000000ll;  // about two seconds
+constexpr long long kSpinClocks = 4000000000ll;  // a wait's limit, about two seconds
 
 // Unpacked rows of a matrix (device), 32 rows per slice.
 struct Rows {
@@ -465,7 +467,7 @@ __device__ __forceinline__ unsigned long long load_acquire(const volatile unsign
 // With FENCE, what the blocks wrote before the call can be read after it;
 // without, only the sum passes between them.
 template <class A, bool FENCE, class Then>
-__device__ __forceinline__ bool grid_sum(A mine, ResState* st, unsigned phase, Then then) {
+__device__ __forceinline__ bool grid_sum(A mine, ResState* st, unsigned phase, long long limit, Then then) {
   constexpr bool kWide = sizeof(A) == 8;
   __shared__ A parts[kResThreads];
   // the two sums of an iteration have words of their own: a block publishes
@@ -487,12 +489,16 @@ __device__ __forceinline__ bool grid_sum(A mine, ResState* st, unsigned phase, T
     const volatile unsigned long long* const w = word + kResWords * threadIdx.x;
     unsigned long long lo = w[0], hi = kWide ? w[1] : phase;
     const long long t0 = clock64();
+    bool over = false;
     while ((unsigned)lo != phase || (unsigned)hi != phase) {
-      if (clock64() - t0 > kSpinClocks || *(volatile int*)&st->status) {
+      // given up only if the words, read after the limit has passed, are not
+      // there (the clock runs on while the whole process is suspended)
+      if (over) {
         st->status = 1;
         bad = true;
         break;
       }
+      over = clock64() - t0 > limit || *(volatile int*)&st->status;
       lo = w[0];
       if (kWide) hi = w[1];
     }
@@ -555,7 +561,8 @@ __device__ __forceinline__ typename T::A row_dot(int len, const int32_t* __restr
 template <class T>
 __global__ void __launch_bounds__(kResThreads, kResPerSm)
     k_cg_resident(int64_t n, const Rows rows, typename T::X* x, typename T::X* r, typename T::X* p, typename T::X* q,
-                  double* scal, ResState* st, double stop, double fall, int every, int held, int max_it) {
+                  double* scal, ResState* st, double stop, double fall, int every, int held, int max_it,
+                  long long limit) {
   using A = typename T::A;
   using X = typename T::X;
   const int64_t nrows = (int64_t)gridDim.x * kResThreads;  // rows of one round
@@ -632,7 +639,7 @@ __global__ void __launch_bounds__(kResThreads, kResPerSm)
       prod = fma((A)pn, (A)qn, prod);
     }
     prod = res_block_sum<A>(prod);
-    if (!grid_sum<A, false>(prod, st, ++phase, [&](double sum) {
+    if (!grid_sum<A, false>(prod, st, ++phase, limit, [&](double sum) {
           pq = sum;
           alpha = sum != 0.0 ? rho / sum : 0.0;
           alpha_x = (X)alpha;
@@ -658,7 +665,7 @@ __global__ void __launch_bounds__(kResThreads, kResPerSm)
       s = fma((A)ri, (A)ri, s);
     }
     s = res_block_sum<A>(s);
-    if (!grid_sum<A, true>(s, st, ++phase, [&](double sum) {
+    if (!grid_sum<A, true>(s, st, ++phase, limit, [&](double sum) {
           beta = rho != 0.0 ? sum / rho : 0.0;
           beta_x = (X)beta;
           rho = sum;
@@ -693,6 +700,7 @@ struct ResLaunch {
   int blocks = 0;  // 0: the handle's iterations run as separate kernels
   int held = 0;    // rows per thread whose p, q and x fit the shared memory
   size_t smem = 0;
+  long long limit = kSpinClocks;
   Rows rows{};
 };
 
@@ -765,7 +773,8 @@ cudaError_t launch_resident(const ResLaunch& l, int64_t n, T* x, T* r, T* p, T* 
                             double stop, double fall, int every, int steps, cudaStream_t s) {
   Rows rows = l.rows;
   int held = l.held;
-  void* args[] = {&n, &rows, &x, &r, &p, &q, &scal, &res, &stop, &fall, &every, &held, &steps};
+  long long limit = l.limit;
+  void* args[] = {&n, &rows, &x, &r, &p, &q, &scal, &res, &stop, &fall, &every, &held, &steps, &limit};
   cudaError_t e = cudaMemsetAsync(res, 0, res_bytes(l.blocks), s);
   if (e == cudaSuccess) e = cudaLaunchCooperativeKernel(l.kern, dim3((unsigned)l.blocks), dim3(kResThreads), args, l.smem, s);
   return e;
@@ -832,8 +841,14 @@ struct UnpackedRows {
 };
 
 // The resident kernel, launched for at most kResIterations iterations at a
-// time, until sqrt(rho) <= stop or max_it.
+// time, until sqrt(rho) <= stop or max_it. SPC5_ETIMEOUT: it was refused or gave
+// up (the caller of cg_solve starts again without it).
 constexpr int kResIterations = 4096;
+
+spc5_status refused(cudaError_t e) {
+  cudaGetLastError();
+  return fail(SPC5_ETIMEOUT, std::string("cg: resident iterations: ") + cudaGetErrorName(e));
+}
 
 template <class T>
 spc5_status cg_resident_loop(const ResLaunch& l, int64_t n, T* x, T* r, T* p, T* q, double* scal, ResState* res,
@@ -842,7 +857,8 @@ spc5_status cg_resident_loop(const ResLaunch& l, int64_t n, T* x, T* r, T* p, T*
   while (*iters < max_it) {
     const int steps = max_it - *iters < kResIterations ? max_it - *iters : kResIterations;
     cudaError_t e = launch_resident<T>(l, n, x, r, p, q, scal, res, stop, 0.0, 1, steps, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(host_scal, scal, sizeof(double) * S_COUNT, cudaMemcpyDeviceToHost, s);
+    if (e != cudaSuccess) return refused(e);
+    e = cudaMemcpyAsync(host_scal, scal, sizeof(double) * S_COUNT, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(e, "cg: resident iterations");
     if (host_scal[S_STATUS] != 0.0) return fail(SPC5_ETIMEOUT, "cg: a grid barrier gave up");
@@ -918,10 +934,9 @@ spc5_status cg_loop(const spc5_matrix* M, T* x, T* r, T* p, T* q, T* w, int64_t 
   return st;
 }
 
-}  // namespace
-
-spc5_status cg_impl(const spc5_matrix* A, const spc5_matrix* L, const double* b, double* x, const spc5_cg_opts* o,
-                    spc5_cg_info* info, cudaStream_t user) {
+// One solve; `resident` allows the resident kernel.
+spc5_status cg_solve(const spc5_matrix* A, const spc5_matrix* L, const double* b, double* x, const spc5_cg_opts* o,
+                     spc5_cg_info* info, cudaStream_t user, bool resident) {
   const int64_t n = A->n;
   // vector kernels: grid-stride, at most kVecBlocksPerSm CTAs per SM (each
   // CTA adds one partial and one ticket to the reductions)
@@ -995,8 +1010,9 @@ spc5_status cg_impl(const spc5_matrix* A, const spc5_matrix* L, const double* b,
   ResLaunch lres;
   UnpackedRows unpacked;
   unsigned long long slots = 0;
-  if (M->nseg == 0 && M->I > 0) {
+  if (resident && M->nseg == 0 && M->I > 0) {
     lres = M->vt == SPC5_F64 ? resident_kernel<F64>(n) : M->vt == SPC5_F32 ? resident_kernel<F32>(n) : resident_kernel<BF16>(n);
+    if (o->wait_us > 0) lres.limit = 2000ll * o->wait_us;  // clocks: at most 2.07 per nanosecond
     if (lres.blocks > 0) {
       e = unpacked.count(M, s);
       if (e == cudaSuccess) e = cudaMemcpyAsync(&slots, unpacked.words.p, sizeof(slots), cudaMemcpyDeviceToHost, s);
@@ -1070,7 +1086,7 @@ spc5_status cg_impl(const spc5_matrix* A, const spc5_matrix* L, const double* b,
         // on the stream: the host looks once per stretch
         const int steps = max_it - info->inner_total < kResIterations ? max_it - info->inner_total : kResIterations;
         e = launch_resident<float>(lres, n, x32, r32, p32, q32, scal, res, stop, kReliableDelta, every, steps, s);
-        if (e != cudaSuccess) return cuda_fail(e, "cg: resident iterations");
+        if (e != cudaSuccess) return refused(e);
       } else {
         const double target = kReliableDelta * rn_upd > 0.5 * stop ? kReliableDelta * rn_upd : 0.5 * stop;
         st = cg_loop<float, float>(L, x32, r32, p32, q32, w32, n, scal, part32, nb, ticket, lres, res, target,
@@ -1166,6 +1182,14 @@ spc5_status cg_impl(const spc5_matrix* A, const spc5_matrix* L, const double* b,
   info->rel_residual = sqrt(hs[S_NORM]) / bnorm;
   info->converged = info->rel_residual <= tol ? 1 : 0;
   return SPC5_OK;
+}
+
+}  // namespace
+
+spc5_status cg_impl(const spc5_matrix* A, const spc5_matrix* L, const double* b, double* x, const spc5_cg_opts* o,
+                    spc5_cg_info* info, cudaStream_t user) {
+  const spc5_status st = cg_solve(A, L, b, x, o, info, user, true);
+  return st == SPC5_ETIMEOUT ? cg_solve(A, L, b, x, o, info, user, false) : st;
 }
 
 }  // namespace spc5

@@ -40,7 +40,8 @@ class Opts(ctypes.Structure):
 class CgOpts(ctypes.Structure):
     _fields_ = [("tol", ctypes.c_double), ("max_iters", ctypes.c_int32), ("max_outer", ctypes.c_int32),
                 ("inner_tol", ctypes.c_double), ("inner_max_iters", ctypes.c_int32), ("check_every", ctypes.c_int32),
-                ("use_graph", ctypes.c_int32), ("reliable", ctypes.c_int32), ("reserved", ctypes.c_int32 * 4)]
+                ("use_graph", ctypes.c_int32), ("reliable", ctypes.c_int32), ("wait_us", ctypes.c_int32),
+                ("reserved", ctypes.c_int32 * 3)]
 
 
 class CgInfo(ctypes.Structure):

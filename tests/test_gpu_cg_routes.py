@@ -75,3 +75,29 @@ def test_float64_rows_around_the_change_of_route(cuda_device, nz):
     assert info["converged"] and info["rel_residual"] <= 1e-10
     y, again = spc5.cg(M, b, tol=1e-10, use_graph=True)
     assert again == info and torch.equal(x, y)
+
+
+@pytest.mark.parametrize("inner,reliable,every", [(None, 0, 90), (torch.bfloat16, 0, 90), (torch.float32, 1, 8)])
+def test_a_wait_that_runs_out_ends_in_the_separate_kernels(cuda_device, inner, reliable, every):
+    import ctypes
+
+    A = inputs.poisson_shifted(50, 50, 50, seed=4)
+    M = convert(A, torch.float64, 2, 4)
+    L = convert(A, inner, 2, 4) if inner is not None else None
+    b = torch.from_numpy(inputs.vec_uniform(A.n, seed=1)).cuda()
+
+    def solve(wait_us):
+        x = torch.full_like(b, float("nan"))
+        opts, info = spc5.CgOpts(tol=1e-10, check_every=every, reliable=reliable, wait_us=wait_us), spc5.CgInfo()
+        status = spc5.load().spc5_cg(M._h, L._h if L else None, b.data_ptr(), x.data_ptr(), ctypes.byref(opts),
+                                     ctypes.byref(info), None)
+        assert status == spc5.OK and info.converged and info.rel_residual <= 1e-10
+        return x, info
+
+    x, info = solve(0)
+    _, late = solve(1)
+    if not reliable:
+        assert info.iterations % every != 0  # the resident kernel stops at the tolerance
+        assert late.iterations % every == 0 and late.iterations > 0  # the separate ones are looked at after 90
+    y, again = solve(0)  # the library is as it was
+    assert torch.equal(x, y) and again.iterations == info.iterations
