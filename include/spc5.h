@@ -279,8 +279,8 @@ spc5_status spc5_device_peaks(double* hbm_gbs_out, int* sm_count_out, int* sm_cl
  * returning them to the driver; see spc5_pool_trim. */
 spc5_status spc5_destroy(spc5_handle h);
 
-/* spc5_pool_trim - return the memory the library's handle pools keep for
- * reuse to the driver (the arrays of live handles stay). No device work. */
+/* spc5_pool_trim - return the memory the library's pools (handles, scratch,
+ * solves) keep for reuse to the driver (the arrays of live handles stay). No device work. */
 spc5_status spc5_pool_trim(void);
 
 /* spc5_last_error - message of the last failed call on this host thread. */
@@ -535,8 +535,14 @@ typedef struct {
  *            iteration starts from x = 0).
  *   info     receives iteration counts and the true relative residual.
  * Dot products reduce in a fixed order (run-to-run reproducible). Allocates
- * its workspace (a few vectors); synchronises `stream`. Returns SPC5_OK also
- * when the tolerance was not reached (see info->converged).
+ * its workspace: four float64 vectors of n entries, with A_inner five float32
+ * ones, and for the resident kernel the unpacked rows of the matrix it iterates
+ * with - up to three times nnz + 65536 entries of 4 bytes and a value each; where
+ * the rows are more uneven, or the device has no room for them, the iterations run
+ * as separate kernels. The workspace comes from a memory pool of the library's
+ * own, which keeps up to 1 GiB of it for the next solve (see spc5_pool_trim).
+ * Synchronises `stream`. Returns SPC5_OK also when the tolerance was not
+ * reached (see info->converged).
  */
 spc5_status spc5_cg(spc5_handle A, spc5_handle A_inner, const double* b_d, double* x_d, const spc5_cg_opts* opt,
                     spc5_cg_info* info, spc5_stream_t stream);

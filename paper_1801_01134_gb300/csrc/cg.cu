@@ -731,17 +731,20 @@ ResLaunch resident_kernel(int64_t n) {
   return l;
 }
 
-// workspace from the library's pool, in the order of the solve's stream (a
-// dozen cudaMalloc / cudaFree pairs of a few MB took about a millisecond)
+// workspace from the library's pool for solves, in the order of the solve's
+// stream (a dozen cudaMalloc / cudaFree pairs of a few MB took about a
+// millisecond)
 struct Buf {
   void* p = nullptr;
   cudaStream_t s = nullptr;
-  ~Buf() {
-    if (p) cudaFreeAsync(p, s);
-  }
+  ~Buf() { release(); }
   cudaError_t alloc(size_t bytes, cudaStream_t st) {
     s = st;
-    return pool_alloc(&p, bytes, st);
+    return solve_alloc(&p, bytes, st);
+  }
+  void release() {
+    if (p) cudaFreeAsync(p, s);
+    p = nullptr;
   }
 };
 
@@ -819,6 +822,10 @@ struct UnpackedRows {
     SPC5_CASE(8, 4) SPC5_CASE(8, 8) SPC5_CASE(8, 16)
 #undef SPC5_CASE
     return cudaGetLastError();
+  }
+
+  void release() {
+    for (Buf* b : {&words, &len, &off, &col, &val}) b->release();
   }
 
   // second pass; false where the rows are too uneven (or the memory too short)
@@ -1030,7 +1037,10 @@ spc5_status cg_solve(const spc5_matrix* A, const spc5_matrix* L, const double* b
     info->converged = 1;
     return SPC5_OK;
   }
-  if (lres.blocks > 0 && !unpacked.fill(M, slots, s, &lres.rows)) lres.blocks = 0;
+  if (lres.blocks > 0 && !unpacked.fill(M, slots, s, &lres.rows)) {
+    unpacked.release();
+    lres.blocks = 0;
+  }
   const double stop = tol * bnorm;
   double rn_true = -1.0;  // the returned x's residual norm, once a solver has computed it
   spc5_status st = SPC5_OK;
