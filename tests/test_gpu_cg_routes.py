@@ -101,3 +101,71 @@ def test_a_wait_that_runs_out_ends_in_the_separate_kernels(cuda_device, inner, r
         assert late.iterations % every == 0 and late.iterations > 0  # the separate ones are looked at after 90
     y, again = solve(0)  # the library is as it was
     assert torch.equal(x, y) and again.iterations == info.iterations
+
+
+@pytest.mark.parametrize("inner,reliable", [(None, False), (torch.float32, False), (torch.float32, True), (torch.bfloat16, True)])
+def test_graph_and_plain_agree_bitwise_with_long_intervals(cuda_device, inner, reliable):
+    # intervals of more than two blocks take the segment path, so the iterations run as separate
+    # kernels: captured once and replayed (over all reliable updates), or launched one by one
+    A = inputs.poisson_shifted(21, 20, 19, seed=4)
+    kw = dict(long_blocks=2, seg_blocks=3)
+    M = convert(A, torch.float64, 2, 4, **kw)
+    L = convert(A, inner, 2, 4, **kw) if inner is not None else None
+    assert M.arrays().nsegments > 0 and (L is None or L.arrays().nsegments > 0)
+    b = torch.from_numpy(inputs.vec_uniform(A.n, seed=1)).cuda()
+    plain, info = spc5.cg(M, b, A_inner=L, tol=1e-10, reliable=reliable)
+    graph, again = spc5.cg(M, b, A_inner=L, tol=1e-10, reliable=reliable, use_graph=True)
+    assert info["converged"] and again == info and torch.equal(plain, graph)
+    assert not reliable or info["outer"] >= 2
+
+
+def test_graph_and_plain_agree_bitwise_with_uneven_rows(cuda_device):
+    # rows too uneven to lie side by side, none of them long
+    n, hub = 40000, 60
+    rows = [[0] + list(range(1, hub))] + [[0, i] if i < hub else [i] for i in range(1, n)]
+    rowptr = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int64)
+    cols = np.concatenate([np.asarray(r, np.int32) for r in rows])
+    row = np.repeat(np.arange(n), np.diff(rowptr))
+    A = inputs.CSR(n, n, rowptr, cols, np.where(cols == row, np.where(row == 0, 2.0 * hub, 2.0), 0.5))
+    b = torch.from_numpy(inputs.vec_uniform(n, seed=1)).cuda()
+    for kw in ({}, {"A_inner": convert(A, torch.float32, 1, 4), "reliable": True}):
+        M = convert(A, torch.float64, 1, 4)
+        assert M.arrays().nsegments == 0
+        x, info = spc5.cg(M, b, tol=1e-10, **kw)
+        y, again = spc5.cg(M, b, tol=1e-10, use_graph=True, **kw)
+        assert info["converged"] and again == info and torch.equal(x, y)
+
+
+@pytest.mark.parametrize("r,c", [(1, 4), (2, 4), (4, 8)])
+def test_block_matrix(cuda_device, r, c):
+    # dense 3 x 3 blocks around a band, symmetric and dominant: float64, and both precisions inside
+    nb, bs = 700, 3
+    rng = np.random.default_rng(5)
+    pairs = {(i, i) for i in range(nb)}
+    for i in range(nb):
+        for j in rng.integers(max(0, i - 30), min(nb, i + 30), 6):
+            pairs |= {(i, int(j)), (int(j), i)}
+    D = {}
+    for i, j in sorted(pairs):
+        if i <= j:
+            B = rng.uniform(-1, 1, (bs, bs))
+            D[i, j], D[j, i] = (B, B.T) if i < j else (B + B.T, B + B.T)
+    dense_rows, cols = [[] for _ in range(nb * bs)], [[] for _ in range(nb * bs)]
+    for (i, j), B in sorted(D.items()):
+        for a in range(bs):
+            dense_rows[i * bs + a].extend(B[a])
+            cols[i * bs + a].extend(range(j * bs, j * bs + bs))
+    rowptr = np.concatenate([[0], np.cumsum([len(x) for x in cols])]).astype(np.int64)
+    ci, vals = np.concatenate(cols).astype(np.int32), np.concatenate(dense_rows)
+    row = np.repeat(np.arange(nb * bs), np.diff(rowptr))
+    off = np.zeros(nb * bs)
+    np.add.at(off, row, np.abs(vals))
+    vals = np.where(ci == row, off[row] + 1.0, vals)
+    A = inputs.CSR(nb * bs, nb * bs, rowptr, ci, vals)
+    b = inputs.vec_uniform(A.n, seed=1)
+    bd = torch.from_numpy(b).cuda()
+    M = convert(A, torch.float64, r, c)
+    for kw in ({}, {"A_inner": convert(A, torch.float32, r, c), "reliable": True}, {"A_inner": convert(A, torch.bfloat16, r, c)}):
+        x, info = spc5.cg(M, bd, tol=1e-10, **kw)
+        res = b - np.bincount(row, vals * x.cpu().numpy()[ci], A.n)
+        assert info["converged"] and np.linalg.norm(res) <= 1.0001e-10 * np.linalg.norm(b)
