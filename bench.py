@@ -13,7 +13,9 @@ before every product. value = sum(2 nnz) / sum(kernel time) in GFLOP/s
 
 Also reported on the same line: the plain CSR kernel on the same GPU, the
 float32 form, an end-to-end figure with host buffers, the roofline of the
-dominant kernel and the CPU oracle timed on the host cores.
+dominant kernel and the CPU oracle timed on the host cores. The line stays
+short (a reader that keeps the end of the output keeps all of it); the sections
+in full, with every shape's sweep, go to stderr.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 """
@@ -71,8 +73,9 @@ def parse():
                    help="measure the float64 / float32 multiply-add rates (1..32 active lanes) and the copy ceiling")
     p.add_argument("--cg-n", type=int, default=96, help="grid edge of the CG profiling matrix")
     p.add_argument("--cg-every", type=int, default=8)
-    p.add_argument("--cg-graph", type=int, default=1)
-    p.add_argument("--cg-variant", type=int, default=18, help="kernel variant of the inner (float32) CG handle")
+    p.add_argument("--cg-graph", type=int, default=1, help="replay captured iterations where they run as separate kernels")
+    p.add_argument("--cg-variant", type=int, default=18, help="kernel variant of the inner (float32) CG handle (its float64 product and the separate "
+                   "kernels take it; the resident iterations read unpacked rows)")
     p.add_argument("--cg-shape", default="2x4", help="block shape of the CG profiling handles")
     p.add_argument("--cg-inner-tol", type=float, default=0.0, help="inner tolerance of the mixed CG (0 = default)")
     return p.parse_args()
@@ -348,6 +351,42 @@ def matrix_entry(p, tlist, key, hbm_peak, roofline=None):
     if roofline is not None:
         e["roofline"] = roofline
     return e
+
+
+LINE_MAX = 7000  # characters of the printed line
+
+
+def short_line(line: dict) -> dict:
+    """The printed line: everything but the sections as it is, of each section the
+    figures it stands for."""
+    def per(ms):
+        return {m["matrix"]: {k: m[k] for k in ("shape", "variant", "ms", "gflops", "hbm_frac")} for m in ms}
+
+    def csr(c):
+        return {"value": c["value"], "speedup_beta_over_csr": c["speedup_beta_over_csr"],
+                "beta_over_csr": {k: v["beta_over_csr"] for k, v in c["per_matrix"].items()}}
+
+    def cg(c):
+        return {k: (v["ms"], v["iterations"]) for k, v in c.items() if isinstance(v, dict) and "ms" in v}
+
+    out = dict(line)
+    out["roofline"] = {k: v for k, v in line["roofline"].items() if k != "alu_fp64"}
+    alu = line["roofline"].get("alu_fp64")
+    if alu:
+        out["roofline"]["alu_fp64"] = {k: alu[k] for k in ("achieved", "peak", "unit", "frac", "peak_measured", "frac_of_measured")}
+    out["per_matrix"], out["csr"] = per(line["per_matrix"]), csr(line["csr"])
+    for key in ("f32", "bf16"):
+        sec = line[key]
+        out[key] = {"value": sec["value"], "unit": sec["unit"], "hbm_frac": sec["hbm_frac"], "csr": csr(sec["csr"]),
+                    "gflops": {m["matrix"]: m["gflops"] for m in sec["per_matrix"]}}
+    out["cg"] = {"ms_and_iterations": cg(line["cg"]), "shifted": cg(line["cg"]["shifted"])}
+    out["spmm_f32"] = {name: {k: (v["ms"], v["gflops"]) for k, v in sec.items() if isinstance(v, dict) and "gflops" in v}
+                       for name, sec in line["spmm_f32"].items() if isinstance(sec, dict)}
+    out["batch_f32"] = {k: line["batch_f32"][k] for k in ("graph_ms", "gflops_graph", "direct_ms", "speedup_vs_per_matrix")}
+    held = line["selector"].get("held_out", {}) if line["selector"] else {}
+    out["selector"] = {k: v["mean"] for k, v in held.items() if isinstance(v, dict) and "mean" in v}
+    out["sections"] = "in full on stderr"
+    return out
 
 
 # ---------------------------------------------------------------------- SpMM
@@ -1065,7 +1104,8 @@ def main():
         "spmm_f32": spmm_res, "batch_f32": batch_res, "selector": sel_res,
     }
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print("bench: sections in full: " + json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(short_line(line)), flush=True)
     if ws > 1:
         import torch.distributed as dist
 
