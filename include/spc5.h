@@ -490,14 +490,15 @@ typedef struct {
                               convergence rate predicts the stop (between
                               check_every/4 and 8 x check_every apart); 1 reads
                               after every iteration (exact stopping point). A
-                              matrix without long intervals runs its iterations
-                              in one resident kernel, which sees the norm after
-                              each: it stops exactly at the tolerance, and looks
-                              every check_every iterations whether a reliable
-                              update is due                                     [8] */
-  int32_t use_graph;       /* replay the iteration from a captured CUDA graph (a
-                              matrix with long intervals; the resident kernel
-                              needs none)                                       [0: off] */
+                              matrix without long intervals (rows not too uneven;
+                              float64 iterations: up to about three million rows)
+                              runs its iterations in one resident kernel, which
+                              sees the norm after each: it stops exactly at the
+                              tolerance, and looks every check_every iterations
+                              whether a reliable update is due                  [8] */
+  int32_t use_graph;       /* replay the iteration from a captured CUDA graph
+                              where it runs as separate kernels (the resident
+                              kernel needs none)                                [0: off] */
   int32_t reliable;        /* with A_inner: 1 = one float32 CG recurrence with
                               reliable updates (the float64 residual replaces
                               the recurred one whenever its norm fell 10x; no

@@ -1647,7 +1647,7 @@ spc5_status convert_impl(int64_t n, int64_t m, int64_t nnz, const int64_t* rowpt
   int64_t nb = 0, ns = 0;
   spc5_status st = SPC5_OK;
   DeviceBuf marks, wcount, wprefix;  // r = 1: one block-start bit per entry, prefix of the word popcounts
-  DeviceBuf hints;                   // rows of the entry chunks (r = 1 passes, r > 1 value pass)
+  DeviceBuf hints;                   // rows of the entry chunks (r = 1 passes)
   const int64_t eth = (nnz + kEntriesPerThread - 1) / kEntriesPerThread;
   const int64_t nwords = (nnz + 31) / 32;
   const int64_t nhint = (nnz + kHintChunk - 1) / kHintChunk;
