@@ -489,16 +489,17 @@ __device__ __forceinline__ bool grid_sum(A mine, ResState* st, unsigned phase, l
     const volatile unsigned long long* const w = word + kResWords * threadIdx.x;
     unsigned long long lo = w[0], hi = kWide ? w[1] : phase;
     const long long t0 = clock64();
-    bool over = false;
     while ((unsigned)lo != phase || (unsigned)hi != phase) {
-      // given up only if the words, read after the limit has passed, are not
-      // there (the clock runs on while the whole process is suspended)
-      if (over) {
+      if (clock64() - t0 > limit || *(volatile int*)&st->status) {
+        // given up only if the words, read once more, are not there (the clock
+        // runs on while the whole process is suspended)
+        lo = w[0];
+        if (kWide) hi = w[1];
+        if ((unsigned)lo == phase && (unsigned)hi == phase) break;
         st->status = 1;
         bad = true;
         break;
       }
-      over = clock64() - t0 > limit || *(volatile int*)&st->status;
       lo = w[0];
       if (kWide) hi = w[1];
     }
