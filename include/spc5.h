@@ -279,8 +279,8 @@ spc5_status spc5_device_peaks(double* hbm_gbs_out, int* sm_count_out, int* sm_cl
  * returning them to the driver; see spc5_pool_trim. */
 spc5_status spc5_destroy(spc5_handle h);
 
-/* spc5_pool_trim - return the memory the library's pools (handles, scratch,
- * solves) keep for reuse to the driver (the arrays of live handles stay). No device work. */
+/* spc5_pool_trim - return the memory the library's pools (handles, scratch)
+ * keep for reuse to the driver (the arrays of live handles stay). No device work. */
 spc5_status spc5_pool_trim(void);
 
 /* spc5_last_error - message of the last failed call on this host thread. */
@@ -541,7 +541,8 @@ typedef struct {
  * with - up to three times nnz + 65536 entries of 4 bytes and a value each; where
  * the rows are more uneven, or the device has no room for them, the iterations run
  * as separate kernels. The workspace comes from a memory pool of the library's
- * own, which keeps up to 1 GiB of it for the next solve (see spc5_pool_trim).
+ * own; after a solve that may have used more than 1 GiB, the pool keeps no more
+ * than that (see spc5_pool_trim).
  * Synchronises `stream`. Returns SPC5_OK also when the tolerance was not
  * reached (see info->converged).
  */

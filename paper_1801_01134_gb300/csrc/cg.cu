@@ -732,16 +732,15 @@ ResLaunch resident_kernel(int64_t n) {
   return l;
 }
 
-// workspace from the library's pool for solves, in the order of the solve's
-// stream (a dozen cudaMalloc / cudaFree pairs of a few MB took about a
-// millisecond)
+// workspace from the library's pool, in the order of the solve's stream (a
+// dozen cudaMalloc / cudaFree pairs of a few MB took about a millisecond)
 struct Buf {
   void* p = nullptr;
   cudaStream_t s = nullptr;
   ~Buf() { release(); }
   cudaError_t alloc(size_t bytes, cudaStream_t st) {
     s = st;
-    return solve_alloc(&p, bytes, st);
+    return pool_alloc(&p, bytes, st);
   }
   void release() {
     if (p) cudaFreeAsync(p, s);
@@ -852,6 +851,7 @@ struct UnpackedRows {
 // time, until sqrt(rho) <= stop or max_it. SPC5_ETIMEOUT: it was refused or gave
 // up (the caller of cg_solve starts again without it).
 constexpr int kResIterations = 4096;
+constexpr size_t kSolveKeep = 1ull << 30;  // bytes the pool may keep after a solve that may have used more
 
 spc5_status refused(cudaError_t e) {
   cudaGetLastError();
@@ -1199,8 +1199,14 @@ spc5_status cg_solve(const spc5_matrix* A, const spc5_matrix* L, const double* b
 
 spc5_status cg_impl(const spc5_matrix* A, const spc5_matrix* L, const double* b, double* x, const spc5_cg_opts* o,
                     spc5_cg_info* info, cudaStream_t user) {
-  const spc5_status st = cg_solve(A, L, b, x, o, info, user, true);
-  return st == SPC5_ETIMEOUT ? cg_solve(A, L, b, x, o, info, user, false) : st;
+  spc5_status st = cg_solve(A, L, b, x, o, info, user, true);
+  if (st == SPC5_ETIMEOUT) st = cg_solve(A, L, b, x, o, info, user, false);
+  // A large solve's workspace does not stay in the pool: it is several times the
+  // matrix, and the program may not solve again.
+  const spc5_matrix* M = L ? L : A;
+  const double bytes = (L ? 52.0 : 32.0) * (double)A->n + 3.0 * (double)M->nnz * (double)(4 + value_size(M->vt));
+  if (bytes > (double)kSolveKeep) trim_scratch(kSolveKeep);
+  return st;
 }
 
 }  // namespace spc5

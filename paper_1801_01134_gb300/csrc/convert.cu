@@ -837,11 +837,7 @@ std::mutex g_pool_mu;
 // of an arena's freed place leaves it too small for the next arena, and the
 // pool then maps new memory (about a tenth of the conversions of a series
 // paid 5 ms).
-// Solves have a third, which gives back what it holds beyond kSolveKeep once
-// the solve is over: their unpacked rows and vectors are a multiple of the
-// matrix, and the program may not solve again.
-enum PoolKind { kScratchPool = 0, kArenaPool = 1, kSolvePool = 2, kPoolKinds = 3 };
-constexpr uint64_t kSolveKeep = 1ull << 30;
+enum PoolKind { kScratchPool = 0, kArenaPool = 1, kPoolKinds = 2 };
 cudaMemPool_t g_pools[kMaxPoolDevices][kPoolKinds] = {};
 
 cudaError_t handle_pool(cudaMemPool_t* out, PoolKind kind = kScratchPool) {
@@ -858,7 +854,7 @@ cudaError_t handle_pool(cudaMemPool_t* out, PoolKind kind = kScratchPool) {
     cudaMemPool_t p = nullptr;
     e = cudaMemPoolCreate(&p, &props);
     if (e != cudaSuccess) return e;
-    uint64_t keep = kind == kSolvePool ? kSolveKeep : UINT64_MAX;  // UINT64_MAX: never release on synchronisation
+    uint64_t keep = UINT64_MAX;  // never release on synchronisation
     e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
     if (e != cudaSuccess) {
       cudaMemPoolDestroy(p);
@@ -1386,11 +1382,11 @@ cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s) {
   return e;
 }
 
-cudaError_t solve_alloc(void** p, size_t bytes, cudaStream_t s) {
+// the scratch pool gives back what it holds unused beyond `keep` bytes
+cudaError_t trim_scratch(size_t keep) {
   cudaMemPool_t pool = nullptr;
-  cudaError_t e = handle_pool(&pool, kSolvePool);
-  if (e == cudaSuccess) e = cudaMallocFromPoolAsync(p, bytes > 0 ? bytes : 16, pool, s);
-  return e;
+  const cudaError_t e = handle_pool(&pool);
+  return e == cudaSuccess ? cudaMemPoolTrimTo(pool, keep) : e;
 }
 
 void destroy_matrix(spc5_matrix* h) {
