@@ -46,8 +46,10 @@ constexpr int kLists = 15;             // lists of one 8-row group: 8 + 4 + 2 + 
 constexpr int kPiece = 1536;           // entries of a long group's column range, about
 constexpr int kCandidates = 256;       // entries looked at for a range's start
 // queued runs hold at least two of a level's entries, so a thread's nine places
-// give at most five; a carried step queues the first and last run of each list too
-constexpr int kQueue = 4 * 5 * kCntThreads + 2 * kLists + 2;
+// give at most five; a carried step queues the first and last run of each list
+// too, and a list's last entry is queued by itself where it lies within 16 of
+// INT_MAX, which stands behind every list
+constexpr int kQueue = 4 * 5 * kCntThreads + kLists * (kCntRows / 8) + 2 * kLists + 2;
 constexpr int kCntPerSm = 4;           // thread blocks per SM of the persistent grid (50 KB of shared memory each)
 
 struct CountShared {
@@ -150,8 +152,9 @@ __device__ __forceinline__ unsigned row_runs(CountShared& sh, int rows, int tota
       if (d == base) prev = -16;
       sh.row[d] = (uint8_t)r;
       const int32_t after = d + 1 < total ? sh.col[0][d + 1] : INT_MAX;
+      const int32_t next = d + 1 < end ? after : INT_MAX;
       if (apart(prev, c)) {
-        if ((d + 1 < end && !apart(c, after)) || (CARRY && (d == base || d + 1 == end)))
+        if (!apart(c, next) || (CARRY && (d == base || d + 1 == end)))
           runs |= 1u << (d - d0);
         else
           ++single;
@@ -212,7 +215,7 @@ __device__ __forceinline__ unsigned merge_lists(CountShared& sh, int k, int tota
       }
       dst[d] = c;
       if (apart(prev, c)) {
-        if ((d + 1 < end && !apart(c, min(x, y))) || (CARRY && (d == base || d + 1 == end)))
+        if (!apart(c, min(x, y)) || (CARRY && (d == base || d + 1 == end)))
           runs |= 1u << (d - d0);
         else
           ++single;
